@@ -42,6 +42,8 @@ int reduce_blocks_for(long long n);
 size_t pmb_generic_smem(const Geom &g, int precision);
 size_t pmb_fast_smem(const Geom &g);
 size_t np_fast_smem(const Geom &g);
+int pmb_split(const Geom &g, int pair_threads);
+size_t rows_smem(const RowArgs &ra, bool force, bool param_table);
 size_t lps_generic_smem(const Geom &g, int precision, bool dil);
 size_t jvp_smem(const Geom &g, int precision);
 // Per-bond tangent cache (pd_tangent.cu): prepare at a linearisation point,
@@ -113,6 +115,9 @@ struct pd_sim {
     std::vector<float4> htab_a, htab_b;   // host copies (passed as kernel parameters when small)
     int *tile_nbr = nullptr;        // [ntiles * 27]
     int nbr_ok = 0;
+    RowArgs rows[2] = {};           // row-wise passes (pd_rows.cuh): LPS dilatation; PMB or LPS force
+    bool rows_ok = false;
+    std::vector<float4> rows_htab[2];
     uint32_t *box_map = nullptr;    // [paired halo box] neighbour tile + brick code of both points
     int box_edge[3] = {0, 0, 0};    // largest tile origin per axis for which box_map holds
     // CSR
@@ -249,6 +254,78 @@ int pdk::validate_description(const pd_grid *gr, const pd_material *mt, const pd
 {
     if (!gr || !mt || !rn) { set_error("null description"); return PD_EINVAL; }
     return validate(gr, mt, rn);
+}
+
+// Tables of the row-wise passes (pd_rows.cuh): the stencil's rows (dz, dy) cut into
+// segments of 5, 3 and 1 bonds, where a part of the sum ends as well, and the rows that
+// each plane of the box stores.
+static int create_rows(pd_sim *s, const std::vector<int4> &st)
+{
+    const Geom &g = s->g;
+    const Material &mt = s->mat;
+    const bool lps = mt.model == PD_MODEL_LPS;
+    RowArgs ra = {};
+    const int m = g.m, HX = 8 + 2 * m;
+    for (int z = -m; z < 4 + m; ++z) {
+        const int c = z < 0 ? -z : std::max(0, z - 3);
+        int R = 0;
+        while ((R + 1) * (R + 1) + c * c <= m * m) ++R;
+        ra.plane[z + m] = ra.nbox - (m - R) * HX;
+        ra.nbox += (8 + 2 * R) * HX;
+    }
+    ra.parts = lps ? (g.W >= 2 ? 2 : 1) : pmb_split(g, s->run.pair_threads);
+    if (ra.parts > std::min(2, g.W)) return PD_OK;
+    // first stencil entry of the second part: PMB cuts the words at W / 2, LPS at (W + 1) / 2
+    const int cut = ra.parts == 2 ? 32 * (lps ? (g.W + 1) / 2 : g.W / 2) : g.S;
+    auto bits = [](int x) {
+        float f;
+        memcpy(&f, &x, sizeof(f));
+        return f;
+    };
+    for (int which = lps ? 0 : 1; which < 2; ++which) {
+        const float two = which == 0 ? 2.f : 1.f;           // the dilatation's table holds 2 d
+        std::vector<float4> &tab = s->rows_htab[which];
+        for (int k = 0; k < g.S; ++k) {
+            const int4 d = st[k];
+            const double d2 = d.w, rr = sqrt(d2);
+            const double vij = mt.vol_corr && rr > m - 0.5 ? (m + 0.5 - rr) : 1.0;
+            const float dx = two * (float)d.x;
+            if (lps) {
+                tab.push_back(make_float4((float)rr, (float)rr, (float)d2, (float)d2));
+                tab.push_back(make_float4(dx, dx, (float)vij, 0.f));
+            } else {
+                const float R = (float)(rr / vij), C = (float)(d2 / vij);
+                tab.push_back(make_float4((float)d2, (float)d2, R, R));
+                tab.push_back(make_float4(C, C, dx, dx));
+            }
+        }
+        ra.nseg = 0;
+        for (int k = 0; k < g.S;) {
+            if (k == cut) ra.split = ra.nseg;
+            const int end = k < cut ? cut : g.S;
+            int len = 1;        // dx consecutive in one row and part
+            while (len < 5 && k + len < end && st[k + len].z == st[k].z && st[k + len].y == st[k].y &&
+                   st[k + len].x == st[k].x + len)
+                ++len;
+            len -= len == 2 || len == 4;
+            const int off = st[k].x + HX * st[k].y;
+            tab.push_back(make_float4(bits((off & 0xffff) | (st[k].z + m) << 16 | len << 24), bits(k), two * st[k].y,
+                                      two * st[k].z));
+            ++ra.nseg;
+            k += len;
+        }
+        tab.push_back(make_float4(0.f, 0.f, 0.f, 0.f));     // read ahead of the last segment
+        ra.ntab = (int)tab.size();
+        if (rows_smem(ra, lps, false) > SMEM_LIMIT) return PD_OK;
+        float4 *dtab = nullptr;
+        ALLOC(dtab, sizeof(float4) * tab.size());
+        PD_CUDA(cudaMemcpy(dtab, tab.data(), sizeof(float4) * tab.size(), cudaMemcpyHostToDevice));
+        ra.tab = dtab;
+        ra.htab = tab.data();
+        s->rows[which] = ra;
+    }
+    s->rows_ok = true;
+    return PD_OK;
 }
 
 static int create_impl(pd_sim *s)
@@ -567,6 +644,10 @@ static int create_impl(pd_sim *s)
     ALLOC(s->io_dn, sizeof(double) * 2 * 3 * NP);
     ALLOC(s->d_err, sizeof(int));
     ALLOC(s->d_count, sizeof(unsigned long long));
+    if (s->precision == PD_FP32C && g.dim == 3 && g.L == 9 && s->nbr_ok && !np_law) {
+        const int rc = create_rows(s, st);
+        if (rc != PD_OK) return rc;
+    }
     // last, so that it moves no other array of the pool
     if (!box_map.empty()) {
         ALLOC(s->box_map, sizeof(uint32_t) * box_map.size());
@@ -631,6 +712,7 @@ static TileArgs make_args(pd_sim *s, int mode, const float4 *src_hl, const doubl
     a.htab_b = s->htab_b.empty() ? nullptr : s->htab_b.data();
     a.ntab_a = (int)s->htab_a.size();
     a.ntab_b = (int)s->htab_b.size();
+    a.rows = s->rows_ok ? s->rows : nullptr;
     a.tile_nbr = s->tile_nbr;
     a.nbr_ok = s->nbr_ok;
     a.box_map = s->box_map;
@@ -691,6 +773,7 @@ int pdk::sim_pack_info(pd_sim *s, PackInfo *pi)
         a.update_breaking = 0;
         a.split = pi->split;
         a.htab_a = a.htab_b = nullptr;      // the packed bodies read the device tables
+        a.rows = nullptr;
         a.ntab_a = a.ntab_b = 0;
         pi->a[p] = a;
     }

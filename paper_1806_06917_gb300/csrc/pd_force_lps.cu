@@ -18,6 +18,8 @@
 
 namespace pdk {
 
+int launch_rows_lps(const TileArgs &a, const RowArgs &ra, int dil, cudaStream_t st);
+
 size_t lps_fast_smem(const Geom &g, bool dil)
 {
     const size_t n = (size_t)(g.bx + 2 * g.m) * (g.by + 2 * g.m) * (g.bz / 2 + 2 * g.m);
@@ -161,6 +163,8 @@ int launch_lps_args(const TileArgs &a, int precision, int dil, cudaStream_t st)
 {
     const Geom &g = a.g;
     const size_t smem = lps_generic_smem(g, precision, dil);
+    if (precision == PD_FP32C && a.rows && g.ntiles >= (dil ? ROWS_MIN_TILES : ROWS_MIN_TILES_FRC))
+        return launch_rows_lps(a, a.rows[dil ? 0 : 1], dil, st);
     if (precision == PD_FP32C) {
         // dilatation: two pairs per thread from 2^7-point tiles and two stencil words on
         const bool dil2 = dil && g.T >= 128 && g.W >= 2;

@@ -23,6 +23,8 @@
 
 namespace pdk {
 
+int launch_rows_pmb(const TileArgs &a, const RowArgs &ra, cudaStream_t st);
+
 // Paired halo box (float4 {x_A, x_B, y_A, y_B}, plus float2 {z_A, z_B} in 3D)
 // followed by the stencil table of `words` float4 per entry.
 static size_t fast_smem(const Geom &g, int words)
@@ -391,6 +393,13 @@ static int choose_split(const Geom &g, size_t base, int pairs_per_thread = 1)
     return best;
 }
 
+// Ranges of stencil words in which a point pair's bonds are summed (the partial sums
+// added in order), whichever kernel runs: the threads per pair of pmb_fast.
+int pmb_split(const Geom &g, int pair_threads)
+{
+    return pair_threads ? pair_threads : choose_split(g, pmb_fast_smem(g));
+}
+
 // The stencil table as a kernel parameter when it fits one (PTAB_N float4) and
 // the grid runs several waves of tiles: there the bond loops are bound by the
 // shared-memory pipe that the table's reads would share (256^3 PMB step 2.43 ->
@@ -436,6 +445,7 @@ static int launch_fast(const TileArgs &a0, cudaStream_t st)
                   "breaking, or the CTA exceeds its limits", a.split, a.g.W);
         return PD_EINVAL;
     }
+    if (DIM == 3 && !BRK && a.rows && a.g.ntiles >= ROWS_MIN_TILES) return launch_rows_pmb(a, a.rows[1], st);
     return a.split > 1 ? launch_fast_split<DIM, BRK, true>(a, st) : launch_fast_split<DIM, BRK, false>(a, st);
 }
 

@@ -223,7 +223,7 @@ __device__ __forceinline__ void lps_dil_fast2_body(const TileArgs &a, int tile, 
         for (int k = threadIdx.x; k < 3 * S; k += blockDim.x) tab[k] = __ldg(&a.tab_a[k]);
     load_nbr(a, tile, s_nbr);
     __syncthreads();
-    stage_pairs(a, pb, org, tile, s_nbr, P4, P2, true);
+    stage_pairs<!PTAB>(a, pb, org, tile, s_nbr, P4, P2, true);
     __syncthreads();
     // 1/m~ of the tile's points, read by the epilogue (128^3 LPS pass 0.2167 -> 0.2151 ms)
     if (threadIdx.x == 0) l2_prefetch(a.minv32 + (size_t)tile * g.T, 4 * g.T);

@@ -267,6 +267,87 @@ __device__ __forceinline__ void for_pair_slots(const TileArgs &a, const PairBox 
     }
 }
 
+// Stage the box column by column: a thread takes a column (x, y) and loads each of
+// its points that some bond of the tile reaches once (|z| limited by the column's
+// distance from the tile; the pair-wise staging loads the points of shared planes
+// twice), writing the pair (z', z' + 4) when its second point arrives. For 8 x 8 x 8
+// tiles whose halo stays within one tile (nbr_ok). s_plane: where each pair plane
+// starts, or null for the full box. GL points' loads are issued together.
+template <bool FRC, int GL>
+__device__ __forceinline__ void stage_columns(const TileArgs &a, const int4 &org, const Ref32 &ref, const int *s_nbr,
+                                              const int *s_plane, float4 *P4, float2 *P2, float4 *PT)
+{
+    const Geom &g = a.g;
+    const float inv_h = (float)a.inv_h;
+    const float kA = (float)a.A, kB = (float)a.B;                           // LPS: 3K - 5mu, 15mu
+    const int HX = 8 + 2 * g.m;
+    for (int c = threadIdx.x; c < HX * HX; c += blockDim.x) {
+        const int yr = fdiv_small(c, __frcp_rn((float)HX)), xr = c - yr * HX;
+        // lattice units outside the tile in x and y, and the planes past it that leaves
+        const int ox = max(max(g.m - xr, xr - g.m - 7), 0), oy = max(max(g.m - yr, yr - g.m - 7), 0);
+        const int left = g.m * g.m - ox * ox - oy * oy;
+        if (left < 0) continue;
+        const int cm = (int)sfu_sqrt((float)left + 0.5f);
+        const int x = org.x + xr - g.m, y = org.y + yr - g.m;
+        const bool inxy = (unsigned)x < (unsigned)g.nx && (unsigned)y < (unsigned)g.ny;
+        const int k = ((x >> 3) - (org.x >> 3) + 1) + 3 * ((y >> 3) - (org.y >> 3) + 1);
+        const int cxy = brick_code(3, x & 7, y & 7, 0);
+        int base[3];
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            const int t = inxy ? s_nbr[k + 9 * l] : -1;
+            base[l] = t < 0 ? -1 : t * 512 + cxy;
+        }
+        float prev[4][FRC ? 5 : 3];
+        const int np = 8 + 2 * cm;
+        for (int j = 0; j < np; j += 4) {
+#pragma unroll
+            for (int i0 = 0; i0 < 4; i0 += GL) {
+                float4 hi[GL], lo[GL];
+                float mi[GL], th[GL];
+                bool in[GL];
+#pragma unroll
+                for (int i = 0; i < GL; ++i) {
+                    const int zr = j + i0 + i - cm;
+                    const int bs = zr < 0 ? base[0] : zr < 8 ? base[1] : base[2];
+                    in[i] = bs >= 0 && j + i0 + i < np && org.z + zr < g.nz;
+                    hi[i] = lo[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    mi[i] = th[i] = 0.f;
+                    if (in[i]) {
+                        const int zl = zr & 7, s = bs + (((zl | zl << 2 | zl << 4) & 0x49) << 2);
+                        hi[i] = __ldg(&a.src_hl[2 * s]);
+                        lo[i] = __ldg(&a.src_hl[2 * s + 1]);
+                        if (FRC) {
+                            mi[i] = __ldg(&a.minv32[s]);
+                            th[i] = __ldcg(&a.theta32[s]);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < GL; ++i) {
+                    float cur[5];
+                    cur[0] = in[i] ? ((hi[i].x - ref.hx) + (lo[i].x - ref.lx)) * inv_h : 0.f;
+                    cur[1] = in[i] ? ((hi[i].y - ref.hy) + (lo[i].y - ref.ly)) * inv_h : 0.f;
+                    cur[2] = in[i] ? ((hi[i].z - ref.hz) + (lo[i].z - ref.lz)) * inv_h : 0.f;
+                    cur[3] = in[i] ? kA * (th[i] * mi[i]) : 0.f;
+                    cur[4] = kB * mi[i];
+                    float *pv = prev[i0 + i];
+                    const int q = j + i0 + i;
+                    if (q >= 4 && q < np) {
+                        const int zp = q - 4 - cm + g.m;            // pair plane z' = q - 4 - cm
+                        const int at = (s_plane ? s_plane[zp] : zp * HX * HX) + c;
+                        P4[at] = make_float4(pv[0], cur[0], pv[1], cur[1]);
+                        P2[at] = make_float2(pv[2], cur[2]);
+                        if constexpr (FRC) PT[at] = make_float4(pv[3], cur[3], pv[4], cur[4]);
+                    }
+#pragma unroll
+                    for (int d = 0; d < (FRC ? 5 : 3); ++d) pv[d] = cur[d];
+                }
+            }
+        }
+    }
+}
+
 // Stage the paired box of displacements: P4[b] = {xA, xB, yA, yB}, P2[b] = {zA, zB}.
 // s_nbr must be loaded and visible (a __syncthreads after load_nbr). use_map
 // takes the slots from the box map where it holds: fewer instructions per entry,
@@ -275,11 +356,19 @@ __device__ __forceinline__ void for_pair_slots(const TileArgs &a, const PairBox 
 // changes nothing in the one-wave 64^3 PMB step, whose staging waits on memory
 // more than it issues. The coordinate loop is kept apart from for_pair_slots:
 // through it the 2D NP kernel (443^2, m = 20, no map) measured 1 % slower.
+template <bool COLS = false>
 __device__ __forceinline__ void stage_pairs(const TileArgs &a, const PairBox &pb, const int4 &org, int tile,
                                             const int *s_nbr, float4 *P4, float2 *P2, bool use_map)
 {
     const Ref32 ref = tile_ref32(a, tile);
     const float inv_h = (float)a.inv_h;
+    // Columns on grids of two tiles an SM and more (64^3 PMB with breaking 0.0577 -> 0.0553
+    // ms) and in edge tiles, whose other form computes every entry's coordinates (37 x 29 x
+    // 41: 0.0484 -> 0.0469 ms); a single whole tile an SM measured 1-2 % slower with them.
+    if (COLS && a.nbr_ok && a.g.bz == 8 && (a.g.ntiles >= ROWS_MIN_TILES || !box_mapped(a, org))) {
+        stage_columns<false, 1>(a, org, ref, s_nbr, nullptr, P4, P2, nullptr);
+        return;
+    }
     if (use_map && box_mapped(a, org)) {
         for_pair_slots<8>(a, pb, org, s_nbr, true, [&](int b, int sA, int sB) {
             const float4 rA = stage_one(a, a.src_hl, sA, ref, inv_h);

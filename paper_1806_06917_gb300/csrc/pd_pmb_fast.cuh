@@ -288,7 +288,7 @@ __device__ __forceinline__ void pmb_fast_body(const TileArgs &a, int tile, const
     }
     load_nbr(a, tile, s_nbr);
     __syncthreads();
-    stage_pairs(a, pb, org, tile, s_nbr, P4, DIM == 3 ? P2 : nullptr, true);
+    stage_pairs<DIM == 3 && !PTAB>(a, pb, org, tile, s_nbr, P4, DIM == 3 ? P2 : nullptr, true);
     if (tab2) {
         if (k0 < 4 * S) tab[k0] = t0;
         if (k1 < 4 * S) tab[k1] = t1;

@@ -346,6 +346,24 @@ __device__ __forceinline__ void split_bits(double u, float &hi, float &lo)
 
 // ------------------------------------------------------------ kernel args
 
+// Row-wise passes of 3D lattices (pd_rows.cuh): the table holds 2 float4 per stencil
+// entry, then one per segment and one of zeros.
+constexpr int ROWS_PTAB = 280;      // float4 that fit the kernel parameter: m <= 3 (122 entries, 32 segments)
+constexpr int ROWS_PLANES = 20;     // pair planes of the box: 4 + 2m, m <= 8
+// Where the row-wise passes take over: from two tiles per SM on (40^3 PMB, 125 tiles:
+// 0.0201 ms word-wise and 0.0247 row-wise; 64^3, 512 tiles: 0.0493 and 0.0468), the LPS
+// force pass, at 128 registers and two CTAs per SM, from more than one tile per SM on
+// (45 x 37 x 52, 210 tiles: 0.0369 and 0.0342; 33 x 45 x 27 with m = 4, 120 tiles: 0.0389
+// and 0.0427). Below, the word-wise kernels' twice as many threads per tile count.
+constexpr int ROWS_MIN_TILES = 304, ROWS_MIN_TILES_FRC = 153;
+struct RowArgs {
+    const float4 *tab, *htab;       // device table and its host copy
+    int ntab, nseg;                 // float4 of the table, segments
+    int parts, split;               // ranges of stencil words summed apart (1 or 2); first segment of the second
+    int nbox;                       // box entries
+    int plane[ROWS_PLANES];         // entry of plane z' at column (-m, -m): its first rows are not stored
+};
+
 // One POD argument block for every tile kernel.
 struct TileArgs {
     Geom g;
@@ -399,6 +417,7 @@ struct TileArgs {
     // most PTAB_N float4 are passed to the kernels as a parameter, see ParamTab)
     const float4 *htab_a, *htab_b;
     int ntab_a, ntab_b;
+    const RowArgs *rows;        // host: [2] the row-wise passes of this simulation (LPS dilatation; PMB, LPS force), or null
 };
 
 // A stencil table passed as a kernel parameter: the kernel reads it from the
