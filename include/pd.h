@@ -141,7 +141,8 @@ typedef struct {
     int32_t precision;  /* PD_FP32C or PD_FP64 */
     int32_t tile_log2;  /* points per tile = 2^tile_log2 (a Morton brick);
                            0 selects 9, or less when the halo box of a large
-                           horizon would not fit in shared memory; 6..9 */
+                           horizon would not fit in shared memory or (PD_FP64)
+                           the grid has few tiles per SM; 6..9 */
     int32_t integrator; /* PD_INTEGRATOR_VERLET (0) or PD_INTEGRATOR_CD */
     int32_t state;      /* PD_FP32C: PD_STATE_F64 (0) or PD_STATE_DF; must be 0
                            for PD_FP64 */

@@ -115,6 +115,7 @@ struct pd_sim {
     std::vector<float4> htab_a, htab_b;   // host copies (passed as kernel parameters when small)
     int *tile_nbr = nullptr;        // [ntiles * 27]
     int nbr_ok = 0;
+    F64Ent *tab64 = nullptr;        // stencil table of the FP64 path (pd_f64.cu)
     RowArgs rows[2] = {};           // row-wise passes (pd_rows.cuh): LPS dilatation; PMB or LPS force
     bool rows_ok = false;
     std::vector<float4> rows_htab[2];
@@ -394,6 +395,12 @@ static int create_impl(pd_sim *s)
             while (L > 6 && max_smem(g, s->precision, model, false) > SMEM_LIMIT) set_tile(--L);
         }
     }
+    // FP64 passes cost their FP64 instructions, and an SM's tiles share one pipe: from six
+    // tiles per SM on the SMs' shares differ by a few percent, and the finer tiles' staging
+    // adds 1-3 % (64^3 PMB step: 1.84 ms with 512 tiles of 2^9, 1.65 with 1024 of 2^8; 40^3 LPS: 1.01
+    // with 125 tiles of 2^9, 0.90 with 1000 of 2^6)
+    if (s->precision == PD_FP64 && !s->run.tile_log2)
+        for (int L = g.L; L > 6 && (long long)g.tgx * g.tgy * g.tgz < 6 * 152;) set_tile(--L);
     s->tangent_ok = tangent;
 
     // tiles: bricks intersecting the grid, ordered by the Morton code of their origin
@@ -644,6 +651,29 @@ static int create_impl(pd_sim *s)
     ALLOC(s->io_dn, sizeof(double) * 2 * 3 * NP);
     ALLOC(s->d_err, sizeof(int));
     ALLOC(s->d_count, sizeof(unsigned long long));
+    if (s->precision == PD_FP64) {
+        const int HX = g.bx + 2 * g.m, HY = g.by + 2 * g.m;
+        std::vector<F64Ent> tab(g.S);
+        for (int k = 0; k < g.S; ++k) {
+            const int4 d = st[k];
+            const double rr = r0[k], d2 = d.w, v = mt.vol_corr && rr > g.m - 0.5 ? (g.m + 0.5 - rr) : 1.0;
+            F64Ent e = {(double)d.x, (double)d.y, (double)d.z, d2, rr / v, d2 / v, v, d.x + HX * (d.y + HY * d.z), 0};
+            if (mt.model == PD_MODEL_LPS) {
+                e.R = rr;
+                e.C = v;
+            } else if (np_law) {    // S / |d| = p / (d2 |d|), exponent -beta h |d| S^2 = a' p^2, p = d.e; J = 0 at m
+                e.R = d2 < (double)g.m * g.m ? v / (rr * d2) : 0.0;
+                e.C = -mt.psi_beta * g.h * rr / (d2 * d2);
+            }
+            const double near = d2 * mt.s_c * (2.0 + mt.s_c) * (1.0 - 0x1p-16);
+            uint64_t nb;
+            memcpy(&nb, &near, sizeof(nb));
+            e.near = (int)(nb >> 32);
+            tab[k] = e;
+        }
+        ALLOC(s->tab64, sizeof(F64Ent) * g.S);
+        PD_CUDA(cudaMemcpy(s->tab64, tab.data(), sizeof(F64Ent) * g.S, cudaMemcpyHostToDevice));
+    }
     if (s->precision == PD_FP32C && g.dim == 3 && g.L == 9 && s->nbr_ok && !np_law) {
         const int rc = create_rows(s, st);
         if (rc != PD_OK) return rc;
@@ -712,6 +742,7 @@ static TileArgs make_args(pd_sim *s, int mode, const float4 *src_hl, const doubl
     a.htab_b = s->htab_b.empty() ? nullptr : s->htab_b.data();
     a.ntab_a = (int)s->htab_a.size();
     a.ntab_b = (int)s->htab_b.size();
+    a.tab64 = s->tab64;
     a.rows = s->rows_ok ? s->rows : nullptr;
     a.tile_nbr = s->tile_nbr;
     a.nbr_ok = s->nbr_ok;

@@ -12,13 +12,12 @@
 // The weighted volume m~ is computed once at the neighbour build.
 #include <string.h>
 
-#include <type_traits>
-
 #include "pd_lps_fast.cuh"
 
 namespace pdk {
 
 int launch_rows_lps(const TileArgs &a, const RowArgs &ra, int dil, cudaStream_t st);
+int launch_f64_lps(const TileArgs &a, int dil, size_t smem, cudaStream_t st);
 
 size_t lps_fast_smem(const Geom &g, bool dil)
 {
@@ -26,127 +25,6 @@ size_t lps_fast_smem(const Geom &g, bool dil)
     const size_t p2 = ((n + 1) / 2) * sizeof(float4);
     if (dil) return n * sizeof(float4) + p2 + (size_t)g.S * 3 * sizeof(float4);
     return 2 * n * sizeof(float4) + p2 + (size_t)g.S * 3 * sizeof(float4);
-}
-
-// ------------------------------------------------------------------ generic
-
-template <class R>
-__global__ void __launch_bounds__(256) lps_dil_generic(const TileArgs a)
-{
-    using R4 = typename std::conditional<sizeof(R) == 4, float4, double4_32a>::type;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    R4 *box = reinterpret_cast<R4 *>(smem_raw);
-    const Geom &g = a.g;
-    const int m = g.m;
-    const int HX = g.bx + 2 * m, HY = g.by + 2 * m, HZ = g.bz + 2 * m;
-    const int nbox = HX * HY * HZ;
-    const int tile = blockIdx.x;
-    const int4 org = __ldg(&a.tile_org[tile]);
-    if constexpr (sizeof(R) == 4)
-        stage_box32(reinterpret_cast<float4 *>(box), HX, HY, nbox, m, a, org, tile_ref32(a, tile), (float)a.inv_h);
-    else
-        stage_box64(reinterpret_cast<double4_32a *>(box), HX, HY, nbox, m, a, org, tile_ref64(a, tile), a.inv_h);
-    __syncthreads();
-    for (int t = threadIdx.x; t < g.T; t += blockDim.x) {
-        const int lx = t % g.bx, ly = (t / g.bx) % g.by, lz = t / (g.bx * g.by);
-        const int slot = tile * g.T + brick_code(3, lx, ly, lz);
-        if (!(org.x + lx < g.nx && org.y + ly < g.ny && org.z + lz < g.nz)) continue;
-        const int bi = (lx + m) + HX * ((ly + m) + HY * (lz + m));
-        const R4 ui = box[bi];
-        R acc = 0;
-        for (int w = 0; w < g.W; ++w) {
-            const uint32_t word = a.mask[(size_t)w * g.nslots + slot];
-            const int nb = min(32, g.S - 32 * w);
-            for (int b = 0; b < nb; ++b) {
-                if (!((word >> b) & 1u)) continue;
-                const int4 d = __ldg(&a.stencil[32 * w + b]);
-                const R r0 = (R)__ldg(&a.stencil_r0[32 * w + b]);
-                const R4 rj = box[bi + d.x + HX * (d.y + HY * d.z)];
-                const R ex = rj.x - ui.x, ey = rj.y - ui.y, ez = rj.z - ui.z;
-                const R yx = ex + (R)d.x, yy = ey + (R)d.y, yz = ez + (R)d.z;
-                const R q = yx * yx + yy * yy + yz * yz;
-                const R num = ex * ex + ey * ey + ez * ez + (R)2 * ((R)d.x * ex + (R)d.y * ey + (R)d.z * ez);
-                const R e = pdiv1(num, q * prsqrt1(q) + r0);
-                R vij = a.vol_corr ? (R)vol_factor_lattice(m, (double)r0) : (R)1;
-                acc += r0 * vij * e;
-            }
-        }
-        if constexpr (sizeof(R) == 4)
-            a.theta32[slot] = 3.f * a.minv32[slot] * acc;
-        else
-            a.theta64[slot] = 3.0 * acc / a.mtil[slot];
-    }
-}
-
-template <class R>
-__global__ void __launch_bounds__(256) lps_force_generic(const TileArgs a)
-{
-    using R4 = typename std::conditional<sizeof(R) == 4, float4, double4_32a>::type;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const Geom &g = a.g;
-    const int m = g.m;
-    const int HX = g.bx + 2 * m, HY = g.by + 2 * m, HZ = g.bz + 2 * m;
-    const int nbox = HX * HY * HZ;
-    R4 *box = reinterpret_cast<R4 *>(smem_raw);
-    R *boxb = reinterpret_cast<R *>(box + nbox);
-    const int tile = blockIdx.x;
-    const int4 org = __ldg(&a.tile_org[tile]);
-    {
-    const double3 ref = tile_ref64(a, tile);
-    for (int b = threadIdx.x; b < nbox; b += blockDim.x) {
-        int x, y, z;
-        box_coord(b, HX, HY, m, 3, org, x, y, z);
-        int s = slot_at(g, a.tile_lut, x, y, z);
-        double4_32a r = make_double4_32a(0.0, 0.0, 0.0, 0.0);
-        double rb = 0.0;
-        if (s >= 0) {
-            double4_32a d = a.src_d4[s];
-            r.x = (d.x - ref.x) * a.inv_h;
-            r.y = (d.y - ref.y) * a.inv_h;
-            r.z = (d.z - ref.z) * a.inv_h;
-            rb = 1.0 / a.mtil[s];
-            r.w = a.theta64[s] * rb;
-        }
-        reinterpret_cast<double4_32a *>(box)[b] = r;
-        reinterpret_cast<double *>(boxb)[b] = rb;
-    }
-    }
-    __syncthreads();
-    const R A = (R)a.A, B = (R)a.B;
-    for (int t = threadIdx.x; t < g.T; t += blockDim.x) {
-        const int lx = t % g.bx, ly = (t / g.bx) % g.by, lz = t / (g.bx * g.by);
-        const int slot = tile * g.T + brick_code(3, lx, ly, lz);
-        if (!(org.x + lx < g.nx && org.y + ly < g.ny && org.z + lz < g.nz)) continue;
-        const int bi = (lx + m) + HX * ((ly + m) + HY * (lz + m));
-        const R4 ui = box[bi];
-        const R bi_ = boxb[bi];
-        R Fx = 0, Fy = 0, Fz = 0;
-        for (int w = 0; w < g.W; ++w) {
-            const uint32_t word = a.mask[(size_t)w * g.nslots + slot];
-            const int nb = min(32, g.S - 32 * w);
-            for (int b = 0; b < nb; ++b) {
-                if (!((word >> b) & 1u)) continue;
-                const int4 d = __ldg(&a.stencil[32 * w + b]);
-                const R r0 = (R)__ldg(&a.stencil_r0[32 * w + b]);
-                const int bj = bi + d.x + HX * (d.y + HY * d.z);
-                const R4 rj = box[bj];
-                const R ex = rj.x - ui.x, ey = rj.y - ui.y, ez = rj.z - ui.z;
-                const R yx = ex + (R)d.x, yy = ey + (R)d.y, yz = ez + (R)d.z;
-                const R q = yx * yx + yy * yy + yz * yz;
-                const R num = ex * ex + ey * ey + ez * ez + (R)2 * ((R)d.x * ex + (R)d.y * ey + (R)d.z * ez);
-                const R rs = prsqrt1(q);
-                const R e = pdiv1(num, q * rs + r0);
-                const R gg = A * r0 * (ui.w + rj.w) + B * e * (bi_ + boxb[bj]);
-                R wgt = gg * rs;
-                if (a.vol_corr) wgt *= (R)vol_factor_lattice(m, (double)r0);
-                Fx += wgt * yx;
-                Fy += wgt * yy;
-                Fz += wgt * yz;
-            }
-        }
-        const double f[3] = {a.inv_h * (double)Fx, a.inv_h * (double)Fy, a.inv_h * (double)Fz};
-        point_epilogue(a, slot, f, 3, sizeof(R) == 8);
-    }
 }
 
 // ---------------------------------------------------------------- dispatch
@@ -191,9 +69,7 @@ int launch_lps_args(const TileArgs &a, int precision, int dil, cudaStream_t st)
             k<<<g.ntiles, threads, smem, st>>>(a);
         }
     } else {
-        auto k = dil ? lps_dil_generic<double> : lps_force_generic<double>;
-        PD_CUDA(smem_limit(k, smem));
-        k<<<g.ntiles, 256, smem, st>>>(a);
+        return launch_f64_lps(a, dil, smem, st);
     }
     PD_CUDA(cudaGetLastError());
     return PD_OK;

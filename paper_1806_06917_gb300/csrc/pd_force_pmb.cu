@@ -11,7 +11,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <type_traits>
 
 #include "pd_pmb_fast.cuh"
 
@@ -24,6 +23,7 @@
 namespace pdk {
 
 int launch_rows_pmb(const TileArgs &a, const RowArgs &ra, cudaStream_t st);
+int launch_f64_bonds(const TileArgs &a, size_t smem, cudaStream_t st);
 
 // Paired halo box (float4 {x_A, x_B, y_A, y_B}, plus float2 {z_A, z_B} in 3D)
 // followed by the stencil table of `words` float4 per entry.
@@ -39,8 +39,6 @@ static size_t fast_smem(const Geom &g, int words)
 size_t pmb_fast_smem(const Geom &g) { return fast_smem(g, 4); }
 
 size_t np_fast_smem(const Geom &g) { return fast_smem(g, NP_TAB_WORDS(g.dim)); }
-
-// ------------------------------------------------------------------ generic
 
 // ------------------------------------------------------------- NP / LP, FP32C
 
@@ -256,111 +254,6 @@ __global__ void __launch_bounds__(1024, 1) np_fast2(const TileArgs a)
     }
 }
 
-// The FP64 stretch of bond (si, sj) with lattice offset d from the global FP64
-// staging (the FP64 path's u), bitwise the same from both ends of the bond.
-__device__ __forceinline__ double canon_stretch64(const TileArgs &a, int si, int sj, int4 d)
-{
-    const double4_32a ui = a.src_d4[si], uj = a.src_d4[sj];
-    const double ex = __dmul_rn(__dsub_rn(uj.x, ui.x), a.inv_h);
-    const double ey = __dmul_rn(__dsub_rn(uj.y, ui.y), a.inv_h);
-    const double ez = __dmul_rn(__dsub_rn(uj.z, ui.z), a.inv_h);
-    const double dx = d.x, dy = d.y, dz = d.z, d2 = d.w;
-    double num = __dmul_rn(ex, __dadd_rn(__dadd_rn(ex, dx), dx));
-    num = __fma_rn(ey, __dadd_rn(__dadd_rn(ey, dy), dy), num);
-    num = __fma_rn(ez, __dadd_rn(__dadd_rn(ez, dz), dz), num);
-    const double r0 = __dsqrt_rn(d2), r = __dsqrt_rn(__dadd_rn(num, d2));
-    return __ddiv_rn(num, __dmul_rn(r0, __dadd_rn(r, r0)));
-}
-
-// Runtime stencil (any horizon), one point per thread. R = float (FP32C) or
-// double (FP64). Stencil entries come from a.stencil; box dims from a.g.m.
-template <class R>
-__global__ void __launch_bounds__(256) pmb_generic(const TileArgs a)
-{
-    using R4 = typename std::conditional<sizeof(R) == 4, float4, double4_32a>::type;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    R4 *box = reinterpret_cast<R4 *>(smem_raw);
-    const Geom &g = a.g;
-    const int m = g.m;
-    const int HX = g.bx + 2 * m, HY = g.by + 2 * m, HZ = g.dim == 3 ? g.bz + 2 * m : 1;
-    const int nbox = HX * HY * HZ;
-    const int tile = blockIdx.x;
-    const int4 org = __ldg(&a.tile_org[tile]);
-    if constexpr (sizeof(R) == 4) {
-        stage_box32(reinterpret_cast<float4 *>(box), HX, HY, nbox, m, a, org, tile_ref32(a, tile),
-                    (float)a.inv_h);
-    } else {
-        stage_box64(reinterpret_cast<double4_32a *>(box), HX, HY, nbox, m, a, org, tile_ref64(a, tile),
-                    a.inv_h);
-    }
-    __syncthreads();
-
-    const bool brk_on = a.update_breaking && a.s_c > 0.0;
-    const bool np_law = a.model == PD_MODEL_NP || a.model == PD_MODEL_LP;
-    const R s_c = (R)a.s_c;
-    for (int t = threadIdx.x; t < g.T; t += blockDim.x) {
-        const int lx = t % g.bx, ly = (t / g.bx) % g.by, lz = t / (g.bx * g.by);
-        const int slot = tile * g.T + brick_code(g.dim, lx, ly, lz);
-        const bool act = org.x + lx < g.nx && org.y + ly < g.ny && org.z + lz < g.nz;
-        if (!act) continue;
-        const int bi = (lx + m) + HX * ((ly + m) + HY * (g.dim == 3 ? lz + m : 0));
-        const R4 ui = box[bi];
-        R Fx = 0, Fy = 0, Fz = 0;
-        for (int w = 0; w < g.W; ++w) {
-            const uint32_t word = a.mask[(size_t)w * g.nslots + slot];
-            uint32_t nword = word;
-            const int nb = min(32, g.S - 32 * w);
-            for (int b = 0; b < nb; ++b) {
-                if (!((word >> b) & 1u)) continue;
-                const int4 d = __ldg(&a.stencil[32 * w + b]);
-                const R4 rj = box[bi + d.x + HX * (d.y + HY * d.z)];
-                const R ex = rj.x - ui.x, ey = rj.y - ui.y, ez = rj.z - ui.z;
-                if (np_law) {
-                    // NP / LP (Algorithm 1): S = eta.d / |d|^2 in lattice units,
-                    // f += J psi'(|xi| S^2)/(C beta) S d/|d| V_ij (times c V below)
-                    if (d.w >= m * m) continue;                            // J = 0 on the boundary
-                    const R r0 = (R)__ldg(&a.stencil_r0[32 * w + b]);
-                    const R S = ((R)d.x * ex + (R)d.y * ey + (R)d.z * ez) / (R)d.w;
-                    R wgt = S / r0;
-                    if (a.model == PD_MODEL_NP) wgt *= exp(-(R)a.psi_beta * (R)a.h * r0 * S * S);
-                    if (a.vol_corr) wgt *= (R)vol_factor_lattice(m, (double)r0);
-                    Fx += wgt * (R)d.x;
-                    Fy += wgt * (R)d.y;
-                    Fz += wgt * (R)d.z;
-                    continue;
-                }
-                const R yx = ex + (R)d.x, yy = ey + (R)d.y, yz = ez + (R)d.z;
-                const R q = yx * yx + yy * yy + yz * yz;
-                const R num = ex * ex + ey * ey + ez * ez +
-                              (R)2 * ((R)d.x * ex + (R)d.y * ey + (R)d.z * ez);
-                const R r0 = (R)__ldg(&a.stencil_r0[32 * w + b]);
-                const R rs = prsqrt1(q);
-                const R s = pdiv1(num, r0 * (q * rs + r0));
-                bool brk = brk_on && s > s_c;
-                // near s_c (2^-30 relative), decided from both points' global state
-                // in an order that is bitwise symmetric in (i, j), as in canon_break32
-                if (brk_on && fabs((double)s - a.s_c) <= 0x1p-30 * a.s_c) {
-                    const int sj = slot_at(g, a.tile_lut, org.x + lx + d.x, org.y + ly + d.y,
-                                           g.dim == 3 ? org.z + lz + d.z : 0);
-                    brk = sj >= 0 && canon_stretch64(a, slot, sj, d) > a.s_c;
-                }
-                if (brk) {
-                    nword &= ~(1u << b);
-                    continue;
-                }
-                R wgt = s * rs;
-                if (a.vol_corr) wgt *= (R)vol_factor_lattice(m, (double)r0);
-                Fx += wgt * yx;
-                Fy += wgt * yy;
-                Fz += wgt * yz;
-            }
-            if (nword != word) a.mask[(size_t)w * g.nslots + slot] = nword;
-        }
-        const double f[3] = {a.cV * (double)Fx, a.cV * (double)Fy, a.cV * (double)Fz};
-        point_epilogue(a, slot, f, g.dim, sizeof(R) == 8);
-    }
-}
-
 // ---------------------------------------------------------------- dispatch
 
 // Shared memory of pmb_fast / np_fast (base) with the stencil split over
@@ -502,11 +395,7 @@ int launch_pmb_args(const TileArgs &a, int precision, cudaStream_t st)
         if (g.dim == 3) return brk ? launch_fast<3, true>(a, st) : launch_fast<3, false>(a, st);
         return brk ? launch_fast<2, true>(a, st) : launch_fast<2, false>(a, st);
     }
-    const size_t smem = pmb_generic_smem(g, precision);
-    PD_CUDA(smem_limit(pmb_generic<double>, smem));
-    pmb_generic<double><<<g.ntiles, 256, smem, st>>>(a);
-    PD_CUDA(cudaGetLastError());
-    return PD_OK;
+    return launch_f64_bonds(a, pmb_generic_smem(g, precision), st);
 }
 
 }  // namespace pdk

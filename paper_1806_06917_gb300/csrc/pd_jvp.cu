@@ -18,6 +18,8 @@
 
 namespace pdk {
 
+int launch_f64_jvp(const TileArgs &a, size_t smem, cudaStream_t st);
+
 template <class R>
 __global__ void __launch_bounds__(256) jvp_generic(const TileArgs a)
 {
@@ -107,13 +109,9 @@ size_t jvp_smem(const Geom &g, int precision)
 int launch_jvp_args(const TileArgs &a, int precision, cudaStream_t st)
 {
     const size_t smem = jvp_smem(a.g, precision);
-    if (precision == PD_FP64) {
-        PD_CUDA(smem_limit(jvp_generic<double>, smem));
-        jvp_generic<double><<<a.g.ntiles, 256, smem, st>>>(a);
-    } else {
-        PD_CUDA(smem_limit(jvp_generic<float>, smem));
-        jvp_generic<float><<<a.g.ntiles, 256, smem, st>>>(a);
-    }
+    if (precision == PD_FP64) return launch_f64_jvp(a, smem, st);
+    PD_CUDA(smem_limit(jvp_generic<float>, smem));
+    jvp_generic<float><<<a.g.ntiles, 256, smem, st>>>(a);
     PD_CUDA(cudaGetLastError());
     return PD_OK;
 }

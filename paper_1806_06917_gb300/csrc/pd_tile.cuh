@@ -110,12 +110,51 @@ __device__ __forceinline__ Pk<R, P> pfmas(const Pk<R, P> &a, R k, const Pk<R, P>
     return pfma(a, splat<R, P>(k), c);
 }
 
-// 1/sqrt(q) and a/b: hardware approximations in FP32 (a few ulp), exact
-// rounding in FP64.
+// ------------------------------------------------------------ FP64 helpers
+
+__device__ __forceinline__ double seed_rsqrt(double x)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return y;
+}
+__device__ __forceinline__ double seed_rcp(double x)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return y;
+}
+
+// sqrt(q) for q > 0: one third-order (Halley-type) step from the seed.
+__device__ __forceinline__ double f64_sqrt(double q)
+{
+    const double y = seed_rsqrt(q), z = q * y;
+    const double g = fma(-z, y, 1.0);
+    return fma(z * g, fma(0.375, g, 0.5), z);
+}
+
+// 1 / sqrt(q) the same way.
+__device__ __forceinline__ double f64_rsqrt(double q)
+{
+    const double y = seed_rsqrt(q);
+    const double g = fma(-(q * y), y, 1.0);
+    return fma(y * g, fma(0.375, g, 0.5), y);
+}
+
+// a / b for b in the normal range, third order from the seed.
+__device__ __forceinline__ double f64_div(double a, double b)
+{
+    const double y = seed_rcp(b);
+    const double g = fma(-b, y, 1.0), z = a * y;
+    return fma(z, fma(g, g, g), z);
+}
+
+// 1/sqrt(q) and a/b: hardware approximations in FP32 (a few ulp), the third-order
+// steps above in FP64 (the last bit).
 __device__ __forceinline__ float prsqrt1(float q) { return rsqrtf(q); }
-__device__ __forceinline__ double prsqrt1(double q) { return 1.0 / sqrt(q); }
+__device__ __forceinline__ double prsqrt1(double q) { return f64_rsqrt(q); }
 __device__ __forceinline__ float pdiv1(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double pdiv1(double a, double b) { return a / b; }
+__device__ __forceinline__ double pdiv1(double a, double b) { return f64_div(a, b); }
 
 template <class R, int P>
 __device__ __forceinline__ Pk<R, P> prsqrt(const Pk<R, P> &q)
@@ -364,6 +403,15 @@ struct RowArgs {
     int plane[ROWS_PLANES];         // entry of plane z' at column (-m, -m): its first rows are not stored
 };
 
+// Stencil entry of the all-FP64 passes (pd_f64.cu), in global memory (its warp-uniform
+// reads hit the L1 while the FP64 pipe is busy).
+struct F64Ent {
+    double dx, dy, dz, d2;
+    double R, C, V;         // PMB: r0 / V_ij, r0^2 / V_ij; LPS: r0, V_ij; NP / LP: k, a'; V_ij
+    int off;                // box offset (x extent bx + 2m, y extent by + 2m)
+    int near;               // PMB with s_c: high word of the num below which a bond is far from breaking
+};
+
 // One POD argument block for every tile kernel.
 struct TileArgs {
     Geom g;
@@ -417,6 +465,7 @@ struct TileArgs {
     // most PTAB_N float4 are passed to the kernels as a parameter, see ParamTab)
     const float4 *htab_a, *htab_b;
     int ntab_a, ntab_b;
+    const F64Ent *tab64;        // stencil table of the all-FP64 passes
     const RowArgs *rows;        // host: [2] the row-wise passes of this simulation (LPS dilatation; PMB, LPS force), or null
 };
 
