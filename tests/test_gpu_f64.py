@@ -42,5 +42,5 @@ def test_fp64_np_force_on_both_sides_of_the_series(pd, scale):
     mat = W.Material(model=W.NP, rho=1.0, psi_c=1.0, psi_beta=1.0)
     sim = gpu_sim(pd, grid, mat, pd.PD_FP64, dt=1e-5)
     u = W.random_field(grid, scale * grid.h, seed=3)
-    assert rel_l2(pd.pd_force(sim, u=u), O.internal_force(grid, mat, O.neighbors(grid), u)) <= 1e-10
+    assert rel_l2(pd.pd_force(sim, u=u), O.internal_force(grid, mat, O.neighbors(grid), u)[0]) <= 1e-10
     sim.close()
