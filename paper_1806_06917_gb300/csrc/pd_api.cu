@@ -56,6 +56,10 @@ int launch_tangent_jacobi(const Geom &g, int precision, void *cache, const int *
                           cudaStream_t st);
 int launch_tangent_precond(const Geom &g, int precision, const void *cache, const double *r, double *z,
                            cudaStream_t st);
+int build_tile_lists(const Geom &g, const Material &mat, const Tables &t, const int4 *host_stencil, const int *tile_nbr,
+                     const uint32_t *box_tab, const int *box_cnt, int nbox, BuildOut *out, uint32_t *mask, double *mtil,
+                     float *minv32, double *d_sum_max, cudaStream_t st);
+size_t tile_rows_smem(const Geom &g, int nbox);
 size_t energy_smem(const Geom &g, int precision);
 int pack_stage(const Geom &g, double *const u[3], float4 *hl, double4_32a *d4, cudaStream_t st, bool bits = false);
 int dirichlet_mask(const Geom &g, const uint8_t *kind, double *const v[3], const double *const w[3], int copy,
@@ -119,6 +123,10 @@ struct pd_sim {
     RowArgs rows[2] = {};           // row-wise passes (pd_rows.cuh): LPS dilatation; PMB or LPS force
     bool rows_ok = false;
     std::vector<float4> rows_htab[2];
+    uint32_t *list_tab = nullptr;   // the neighbour build by tile (pd_lists.cu): halo box table, null: by cell list
+    int *list_cnt = nullptr;
+    int list_nbox = 0;
+    std::vector<int4> hstencil;
     uint32_t *box_map = nullptr;    // [paired halo box] neighbour tile + brick code of both points
     int box_edge[3] = {0, 0, 0};    // largest tile origin per axis for which box_map holds
     // CSR
@@ -609,6 +617,37 @@ static int create_impl(pd_sim *s)
             }
             const int n3[3] = {g.nx, g.ny, g.nz};
             for (int c = 0; c < 3; ++c) s->box_edge[c] = n3[c] % dims[c] == 0 ? INT_MAX : n3[c] - 2 * dims[c];
+        }
+    }
+
+    // The halo box by neighbour tile (pd_lists.cu): entry = tile (27) | code << 5 | index among
+    // the box's points of that tile, in code order, << 14
+    s->hstencil = st;
+    if (s->nbr_ok) {
+        const int dims[3] = {g.bx, g.by, g.dim == 3 ? g.bz : 1}, mz = g.dim == 3 ? g.m : 0;
+        const int HX = g.bx + 2 * g.m, HY = g.by + 2 * g.m, HZ = dims[2] + 2 * mz, nbox = HX * HY * HZ;
+        if (nbox < 1 << 16 && tile_rows_smem(g, nbox) + 16384 + 8192 <= SMEM_LIMIT) {
+            std::vector<uint32_t> tab(nbox);
+            std::vector<int> cnt(27, 0), at(27 * 512, -1);      // box entry by tile and code
+            for (int b = 0; b < nbox; ++b) {
+                const int r[3] = {b % HX - g.m, (b / HX) % HY - g.m, b / (HX * HY) - mz};
+                int dt[3], l[3];
+                for (int c = 0; c < 3; ++c) {
+                    dt[c] = r[c] < 0 ? -1 : r[c] / dims[c];
+                    l[c] = r[c] - dt[c] * dims[c];
+                }
+                const int k = (dt[0] + 1) + 3 * (dt[1] + 1) + 9 * (dt[2] + 1);
+                at[512 * k + (int)morton_encode(g.dim, l[0], l[1], l[2])] = b;
+            }
+            for (int k = 0; k < 27; ++k)
+                for (int code = 0; code < g.T; ++code)
+                    if (at[512 * k + code] >= 0)
+                        tab[at[512 * k + code]] = (uint32_t)k | (uint32_t)code << 5 | (uint32_t)cnt[k]++ << 14;
+            ALLOC(s->list_tab, sizeof(uint32_t) * nbox);
+            ALLOC(s->list_cnt, sizeof(int) * 27);
+            PD_CUDA(cudaMemcpy(s->list_tab, tab.data(), sizeof(uint32_t) * nbox, cudaMemcpyHostToDevice));
+            PD_CUDA(cudaMemcpy(s->list_cnt, cnt.data(), sizeof(int) * 27, cudaMemcpyHostToDevice));
+            s->list_nbox = nbox;
         }
     }
 
@@ -1238,14 +1277,20 @@ int pd_build_neighbors(pd_sim *s, void *stream)
     t.slot_of_user = s->slot_of_user;
     t.rank_of_slot = s->rank_of_slot;
     t.slot_of_rank = s->slot_of_rank;
-    rc = build_csr(s->g, t, &s->csr, s->mask, st);
-    if (rc != PD_OK) return rc;
-    if (s->mat.model == PD_MODEL_LPS) {
-        rc = build_weighted_volume(s->g, s->mat, t, s->mask, s->mtil, s->minv32, st);
+    if (s->list_tab) {
+        rc = build_tile_lists(s->g, s->mat, t, s->hstencil.data(), s->tile_nbr, s->list_tab, s->list_cnt, s->list_nbox,
+                              &s->csr, s->mask, s->mtil, s->minv32, s->dout, st);
+        if (rc != PD_OK) return rc;
+    } else {
+        rc = build_csr(s->g, t, &s->csr, s->mask, st);
+        if (rc != PD_OK) return rc;
+        if (s->mat.model == PD_MODEL_LPS) {
+            rc = build_weighted_volume(s->g, s->mat, t, s->mask, s->mtil, s->minv32, st);
+            if (rc != PD_OK) return rc;
+        }
+        rc = build_dt_bound(s->g, s->mat, t, s->mask, s->dout, st);
         if (rc != PD_OK) return rc;
     }
-    rc = build_dt_bound(s->g, s->mat, t, s->mask, s->dout, st);
-    if (rc != PD_OK) return rc;
     double smax = 0.0;
     PD_CUDA(cudaMemcpyAsync(&smax, s->dout, sizeof(double), cudaMemcpyDeviceToHost, st));
     PD_CUDA(cudaStreamSynchronize(st));

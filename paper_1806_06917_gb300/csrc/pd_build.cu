@@ -92,7 +92,7 @@ __global__ void k_scan_apply(const int *in, long long n, const long long *boff, 
 }
 
 // out[0..n] = exclusive prefix sums of in[0..n), out[n] = total.
-static int exclusive_scan(const int *in, long long n, long long *out, cudaStream_t st)
+int exclusive_scan(const int *in, long long n, long long *out, cudaStream_t st)
 {
     const int nb = (int)((n + SCAN_CHUNK - 1) / SCAN_CHUNK);
     long long *bsum = nullptr;
@@ -105,8 +105,7 @@ static int exclusive_scan(const int *in, long long n, long long *out, cudaStream
         PD_CUDA(cudaMemsetAsync(out, 0, sizeof(long long), st));
     }
     cudaError_t e = cudaGetLastError();
-    cudaStreamSynchronize(st);
-    lib_free(bsum, st);
+    lib_free(bsum, st);         // stream-ordered
     if (e != cudaSuccess) return cuda_fail(e, "exclusive_scan");
     return PD_OK;
 }
@@ -124,7 +123,9 @@ __device__ __forceinline__ void slot_coord(const Geom &g, const int4 *tile_org, 
     c[2] = o.z + l[2];
 }
 
-__global__ void k_slots(Geom g, const int4 *tile_org, int *user_of_slot, int *slot_of_user, int *active)
+// With active == null every slot is a point: its rank is the slot itself.
+__global__ void k_slots(Geom g, const int4 *tile_org, int *user_of_slot, int *slot_of_user, int *active,
+                        int *rank_of_slot, int *slot_of_rank)
 {
     const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= g.nslots) return;
@@ -138,7 +139,12 @@ __global__ void k_slots(Geom g, const int4 *tile_org, int *user_of_slot, int *sl
     } else {
         user_of_slot[s] = -1;
     }
-    active[s] = in ? 1 : 0;
+    if (active) {
+        active[s] = in ? 1 : 0;
+    } else {
+        rank_of_slot[s] = (int)s;
+        slot_of_rank[s] = (int)s;
+    }
 }
 
 __global__ void k_ranks(Geom g, const int *active, const long long *scan, int *rank_of_slot, int *slot_of_rank)
@@ -157,17 +163,25 @@ __global__ void k_ranks(Geom g, const int *active, const long long *scan, int *r
 int build_slots(const Geom &g, const Tables &t, int *user_of_slot, int *slot_of_user, int *rank_of_slot,
                 int *slot_of_rank, cudaStream_t st)
 {
+    const int nb = (g.nslots + 255) / 256;
+    if (g.nslots == g.npoints) {
+        k_slots<<<nb, 256, 0, st>>>(g, t.tile_org, user_of_slot, slot_of_user, nullptr, rank_of_slot, slot_of_rank);
+        PD_CUDA(cudaGetLastError());
+        return PD_OK;
+    }
     int *active = nullptr;
     long long *scan = nullptr;
     PD_CUDA(lib_malloc(reinterpret_cast<void **>(&active), sizeof(int) * (size_t)g.nslots, st));
-    PD_CUDA(lib_malloc(reinterpret_cast<void **>(&scan), sizeof(long long) * ((size_t)g.nslots + 1), st));
-    const int nb = (g.nslots + 255) / 256;
-    k_slots<<<nb, 256, 0, st>>>(g, t.tile_org, user_of_slot, slot_of_user, active);
+    cudaError_t e = lib_malloc(reinterpret_cast<void **>(&scan), sizeof(long long) * ((size_t)g.nslots + 1), st);
+    if (e != cudaSuccess) {
+        lib_free(active, st);
+        return cuda_fail(e, "build_slots");
+    }
+    k_slots<<<nb, 256, 0, st>>>(g, t.tile_org, user_of_slot, slot_of_user, active, nullptr, nullptr);
     int rc = exclusive_scan(active, g.nslots, scan, st);
     if (rc == PD_OK) {
         k_ranks<<<nb, 256, 0, st>>>(g, active, scan, rank_of_slot, slot_of_rank);
-        cudaError_t e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        e = cudaGetLastError();
         if (e != cudaSuccess) rc = cuda_fail(e, "build_slots");
     }
     lib_free(active, st);
@@ -435,7 +449,8 @@ int build_csr(const Geom &g, const Tables &t, BuildOut *out, uint32_t *mask, cud
         rc = exclusive_scan(row_count, n, (long long *)out->row_ptr, st);
         if (rc != PD_OK) goto done;
         long long nbonds = 0;
-        if (cudaMemcpy(&nbonds, out->row_ptr + n, sizeof(long long), cudaMemcpyDeviceToHost) != cudaSuccess) {
+        if (cudaMemcpyAsync(&nbonds, out->row_ptr + n, sizeof(long long), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess) {
             rc = cuda_fail(cudaGetLastError(), "row_ptr readback");
             goto done;
         }
