@@ -1931,7 +1931,8 @@ int pd_solve_static(pd_sim *s, const pd_newton_opts *opts, pd_newton_stats *stat
     }
     if ((rc = ensure_cap(s)) != PD_OK) return rc;
     KrylovWork wk{s->nk_basis, s->nk_tmp, s->nk_aux, s->nk_partial, s->nk_dsc, s->cap_stream};
-    KrylovOp op{cached ? nk_apply_cached : nk_apply, s, jacobi ? nk_precond : nullptr};
+    const TanOp tan = cached ? tangent_op(g, s->precision, s->nk_tan, s->user_of_slot, s->bc_kind) : TanOp{};
+    KrylovOp op{cached ? nk_apply_cached : nk_apply, s, jacobi ? nk_precond : nullptr, cached ? &tan : nullptr};
     const unsigned nbs = (unsigned)((g.nslots + 255) / 256);
 
     // the iterate lives in the FP64 slot arrays u; the prescribed values first

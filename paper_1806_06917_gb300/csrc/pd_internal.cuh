@@ -150,10 +150,21 @@ cudaError_t lib_free(void *p, cudaStream_t st);
 int validate_description(const pd_grid *gr, const pd_material *mt, const pd_run *rn);
 
 // Krylov solvers (pd_krylov.cu). Vectors: n FP64 values on the device.
+// The cached tangent operator for kernels that apply it themselves (pd_tangent.cu).
+struct TanOp {
+    int dim, S, nslots, fp64;
+    const void *coef;           // D [S][3 or 6][nslots]
+    const int *nbr;             // [S][nslots]
+    const int *user_of_slot;
+    const uint8_t *kind;
+};
+TanOp tangent_op(const Geom &g, int precision, const void *cache, const int *user_of_slot, const uint8_t *kind);
+
 struct KrylovOp {
     int (*apply)(void *ctx, const double *x, double *y, cudaStream_t st);   // y = A x
     void *ctx;
     int (*precond)(void *ctx, const double *r, double *z, cudaStream_t st); // z = M^-1 r, or null
+    const TanOp *tan;   // the same operator as the cached tangent, or null
 };
 // Device scalars a Krylov solve needs at least (dot results and CG's state).
 constexpr size_t KRYLOV_DSC_MIN = 24;

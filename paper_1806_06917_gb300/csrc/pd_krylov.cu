@@ -12,35 +12,11 @@
 // formed from p.Ap and r.r. The host reads the scalars back once per chunk of
 // iterations (GM_CHUNK Arnoldi steps, CG_CHUNK CG iterations), each chunk
 // replayed as a captured CUDA graph.
-#include <math.h>
-
-#include <algorithm>
 #include <vector>
 
-#include "pd_tile.cuh"
+#include "pd_krylov.cuh"
 
 namespace pdk {
-
-constexpr int KT = 256;               // threads per block
-constexpr int KPER = 8;               // elements per thread in a reduction block
-constexpr int KCHUNK = KT * KPER;     // elements per reduction block
-
-static int kblocks(long long n) { return (int)((n + KCHUNK - 1) / KCHUNK); }
-
-// Fixed-order sum of one value per thread of the block; the result is valid in
-// thread 0.
-__device__ __forceinline__ double block_sum(double v, double *red)
-{
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    __syncthreads();            // red may still be read from a previous call
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < KT / 32; ++w) t += red[w];
-    return t;
-}
 
 // partial[i * nb + b] = sum over block b of V_i . w (V_i = V + i * ldv); grid
 // (nb, k): block (b, i) sums chunk b of vector i, so all k products run at once.
@@ -140,26 +116,11 @@ static int norm2(KrylovCtx &c, const double *x, double *out)
 
 // ------------------------------------------------------------------ GMRES(m)
 
-// Device layout of GMRES's small arrays in dsc (m = restart): the dot results
-// [0, m+1), the Hessenberg matrix H (column-major, (m+1) x m), the rotations cs
-// and sn, the rotated right-hand side g (m+1), the solution y of the small
-// triangular system (m), and the scalars. The host enqueues GM_CHUNK Arnoldi
-// steps at a time and reads back once per chunk; a step after the one that
-// met the target (or broke down) changes nothing that the update of x uses.
-struct GmLayout {
-    int m, H, cs, sn, g, y, sc;
-    __host__ __device__ explicit GmLayout(int m_)
-        : m(m_), H(m_ + 1), cs(H + (m_ + 1) * m_), sn(cs + m_), g(sn + m_), y(g + m_ + 1), sc(y + m_)
-    {
-    }
-    __host__ __device__ int size() const { return sc + 8; }
-};
-enum { GM_TARGET = 0, GM_DONE, GM_K, GM_RES, GM_INVH, GM_ITERS };
 constexpr int GM_CHUNK = 8;
 
 size_t krylov_dsc_doubles(int krylov_gmres_restart)
 {
-    const size_t g = krylov_gmres_restart > 0 ? (size_t)GmLayout(krylov_gmres_restart).size() : 0;
+    const size_t g = krylov_gmres_restart > 0 ? (size_t)GmLayout(krylov_gmres_restart).size() + 1 : 0;   // + the grid form's barrier
     return std::max(g, KRYLOV_DSC_MIN);
 }
 
@@ -183,60 +144,18 @@ __global__ void __launch_bounds__(KT) k_partial_sum_hcol(const double *partial, 
     *h = add ? *h + t : t;
 }
 
-// After dsc[0] = |w|^2: H[j+1, j] = |w|, the previous rotations and a new one on
-// column j, g rotated, the residual estimate |g[j+1]|, the scale 1/|w| for w.
-// The block stages column j and the rotations in shared memory (3 (m + 1)
-// doubles, dynamic) so that the sequential rotation loop of thread 0 does not
-// wait on global loads.
-// |w|^2 is summed here from the nb block partials of k_mdot, in k_partial_sum's
-// fixed order (KT threads).
+// The Givens step of column j with |w|^2 summed from the nb block partials of k_mdot, in
+// k_partial_sum's fixed order (KT threads).
 __global__ void __launch_bounds__(KT) k_gm_step(const double *partial, int nb, double *d, int m, int j)
 {
     extern __shared__ double gs[];
-    __shared__ double red[KT / 32];
-    const GmLayout L(m);
-    double *sc = d + L.sc;
-    {
-        double acc = 0.0;
-        for (int b = threadIdx.x; b < nb; b += KT) acc += partial[b];
-        const double t = block_sum(acc, red);
-        if (threadIdx.x == 0) d[0] = t;
-        __syncthreads();
-    }
-    if (sc[GM_DONE] != 0.0) {
-        if (threadIdx.x == 0) sc[GM_INVH] = 0.0;
-        return;
-    }
-    double *hj = d + L.H + (m + 1) * j;
-    double *hs = gs, *css = gs + (m + 1), *sns = gs + 2 * (m + 1);
-    for (int i = threadIdx.x; i <= j; i += blockDim.x) hs[i] = hj[i];
-    for (int i = threadIdx.x; i < j; i += blockDim.x) {
-        css[i] = d[L.cs + i];
-        sns[i] = d[L.sn + i];
-    }
+    __shared__ double red[KT / 32], s_ww;
+    double acc = 0.0;
+    for (int b = threadIdx.x; b < nb; b += KT) acc += partial[b];
+    const double t = block_sum(acc, red);
+    if (threadIdx.x == 0) d[0] = s_ww = t;
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    const double hn = sqrt(d[0]);
-    double *cs = d + L.cs, *sn = d + L.sn, *g = d + L.g;
-    hs[j + 1] = hn;
-    for (int i = 0; i < j; ++i) {
-        const double t = css[i] * hs[i] + sns[i] * hs[i + 1];
-        hs[i + 1] = -sns[i] * hs[i] + css[i] * hs[i + 1];
-        hs[i] = t;
-    }
-    const double den = hypot(hs[j], hs[j + 1]);
-    cs[j] = den > 0.0 ? hs[j] / den : 1.0;
-    sn[j] = den > 0.0 ? hs[j + 1] / den : 0.0;
-    hs[j] = den;
-    hs[j + 1] = 0.0;
-    for (int i = 0; i <= j + 1; ++i) hj[i] = hs[i];
-    g[j + 1] = -sn[j] * g[j];
-    g[j] = cs[j] * g[j];
-    sc[GM_K] = j + 1;
-    sc[GM_ITERS] += 1.0;
-    sc[GM_RES] = fabs(g[j + 1]);
-    sc[GM_INVH] = hn > 0.0 ? 1.0 / hn : 0.0;
-    if (sc[GM_RES] <= sc[GM_TARGET] || hn == 0.0) sc[GM_DONE] = 1.0;
+    gm_givens(d, m, j, s_ww, gs);
 }
 
 // y = H(0:k, 0:k)^-1 g(0:k), back substitution
@@ -382,7 +301,24 @@ int krylov_gmres(const KrylovOp &op, const double *b, double *x, long long n, in
         const int steps = std::min(m, maxit - stats->iters);
         int k = 0;
         bool done = false;
-        for (int j0 = 0; j0 < steps && !done; j0 += GM_CHUNK) {
+        bool grid = false;
+        if (op.tan && !pc) {
+            rc = gmres_grid(*op.tan, V, n, c.partial, c.dsc, m, steps, st);
+            grid = rc == PD_OK;
+            if (rc != PD_OK && rc != PD_ENOTREADY) return rc;
+            if (grid) {
+                unsigned sy = 0;
+                PD_CUDA(cudaMemcpyAsync(back, c.dsc + L.sc, sizeof(back), cudaMemcpyDeviceToHost, st));
+                PD_CUDA(cudaMemcpyAsync(&sy, c.dsc + L.size(), sizeof(sy), cudaMemcpyDeviceToHost, st));
+                PD_CUDA(cudaStreamSynchronize(st));
+                if (sy >> 31) {   // a wait that ran out
+                    set_error("GMRES: a wait of the grid kernel ran out");
+                    return PD_ETIMEOUT;
+                }
+                k = (int)back[GM_K];
+            }
+        }
+        for (int j0 = 0; j0 < steps && !done && !grid; j0 += GM_CHUNK) {
             const int j1 = std::min(steps, j0 + GM_CHUNK);
             cudaGraphExec_t ge = j1 == std::min(m, j0 + GM_CHUNK) ? chunk_graph(j0) : nullptr;
             if (ge) {
@@ -610,7 +546,7 @@ int krylov_cg(const KrylovOp &op, const double *b, double *x, long long n, int m
     return PD_OK;
 }
 
-size_t krylov_partial_doubles(long long n, int kmax) { return (size_t)kblocks(n) * (kmax + 1); }
+size_t krylov_partial_doubles(long long n, int kmax) { return (size_t)std::max(kblocks(n), GRID_MAX) * (kmax + 1); }
 
 int krylov_norm(const double *x, long long n, KrylovWork &wk, double *out, cudaStream_t st)
 {

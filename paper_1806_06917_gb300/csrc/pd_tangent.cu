@@ -276,6 +276,13 @@ int launch_tangent_prepare(const TileArgs &a, int precision, void *cache, cudaSt
     return PD_OK;
 }
 
+TanOp tangent_op(const Geom &g, int precision, const void *cache, const int *user_of_slot, const uint8_t *kind)
+{
+    const size_t nc = g.dim == 3 ? 6 : 3, r = precision == PD_FP64 ? sizeof(double) : sizeof(float);
+    const int *nbr = reinterpret_cast<const int *>(static_cast<const char *>(cache) + (size_t)g.S * g.nslots * nc * r);
+    return TanOp{g.dim, g.S, g.nslots, precision == PD_FP64, cache, nbr, user_of_slot, kind};
+}
+
 int launch_tangent_apply(const Geom &g, int precision, const void *cache, const int *user_of_slot,
                          const uint8_t *kind, const double *w, double *y, cudaStream_t st)
 {
