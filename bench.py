@@ -61,7 +61,7 @@ ALG_BYTES = {"pmb3": (4.25, 110.0), "pmb2": (4.25, 76.0), "lps_dil": (4.0, 44.0)
 PER_POINT_BYTES = {"pmb3": 179.0, "pmb2": 134.0, "lps_dil": 56.0, "lps_force": 187.0, "np2": 290.0}
 PASS_KERNEL = {"pmb3": "pmb_fast<3, *> (fused force + update)", "pmb2": "pmb_fast<2, *> (fused force + update)",
                "lps_dil": "lps_dil_fast2 (dilatation pass)", "lps_force": "lps_force_fast (force + update pass)",
-               "np2": "np_fast2 (fused force + update, two point pairs per thread)"}
+               "np2": "np_rows (fused force + update, two point pairs per thread by stencil rows)"}
 FALLBACK_HBM_GBS = 6800.0
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of

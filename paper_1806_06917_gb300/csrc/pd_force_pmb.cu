@@ -11,13 +11,18 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "pd_pmb_fast.cuh"
 
-// Unroll depth of the NP / LP bond loops (8 measured the same as 4 on the 443^2,
-// m = 20 step: 0.1553 ms per launch).
+// Unroll depth of np_fast's bond loops.
 #ifndef PD_NP_UNROLL
 #define PD_NP_UNROLL PD_UNROLL
+#endif
+// Bonds of a row unrolled in np_rows (443^2, m = 20: 0.1338 ms with 4, 0.1323 with 8, 0.1325
+// with 12).
+#ifndef PD_NP_ROW
+#define PD_NP_ROW 8
 #endif
 
 namespace pdk {
@@ -143,114 +148,217 @@ __global__ void __launch_bounds__(SPLIT ? 1024 : 256, SPLIT ? 1 : PD_MINBLOCKS) 
     }
 }
 
-// 2D wide horizons: each thread owns two point pairs, t and t + T/4 (by/4 box
-// rows apart, the constant offset dbi), so that every table entry read from
-// shared memory serves four points: per 32-lane step 2 broadcast table loads
-// and 2 gathers move 128 bonds, against 2 + 1 for 64 bonds with one pair. The
-// shared-memory data pipe bounds np_fast at m = 20; the arithmetic is np_word's.
+// 2D wide horizons: each thread owns two point pairs adjacent in x, and walks each row of
+// the stencil with the box column of its second pair at one bond kept as that of its first
+// at the next: a bond of four points takes one gather and the entry's dx, k and a' (dy is
+// the row's), 8 shared-memory wavefronts a 32-lane step against 12 with two pairs T / 4
+// apart in y. The box is stored as its even columns and then its odd ones, so that a
+// gather's lanes are 16 bytes apart and the columns of a row come from the two halves in
+// turn at constant offsets. What bounds it: the packed FP32 pipe, 40 cycles a step and
+// sub-partition (50,000 cycles of a tile's 68,000 in its bonds, alone on its SM, at m = 20);
+// around the bonds, 8,000 cycles for masks and addresses, 9,000 of staging (19,000 with each
+// point staged by both of its pairs from a Morton order read row by row and a table of tiles
+// in global memory) and 7,000 of update (12,000 by a quarter of the threads), which a younger
+// CTA hardly gets on with while an older one has bonds. 443^2, m = 20 (392 tiles on 304
+// slots): 0.143 -> 0.132 ms a step. The arithmetic is np_word's, bond by bond.
+//
+// Bonds [k, kend) of the stencil, which one word holds if MASKED (c0..c3: its masks of the
+// four points, from bit 0). A row ends at the disk's edge or before the point itself.
 template <bool MASKED, bool LINEAR>
-__device__ __forceinline__ void np_word2(const float4 *tw, int nb, const float4 *P4, int bi, int dbi,
-                                         float2 nux0, float2 nuy0, float2 nux1, float2 nuy1, uint32_t c0,
-                                         uint32_t c1, uint32_t c2, uint32_t c3, float2 &Fx0, float2 &Fy0,
-                                         float2 &Fx1, float2 &Fy1)
+__device__ __forceinline__ void np_row_bonds(const float4 *tab, int m, int k, int kend, const float4 *P4, int half, int bi,
+                                             float2 nux0, float2 nuy0, float2 nux1, float2 nuy1, uint32_t c0,
+                                             uint32_t c1, uint32_t c2, uint32_t c3, float2 &Fx0, float2 &Fy0,
+                                             float2 &Fx1, float2 &Fy1)
 {
-PD_PRAGMA_UNROLL(PD_NP_UNROLL)
-    for (int b = 0; b < nb; ++b) {
-        const float4 ta = tw[2 * b], tb = tw[2 * b + 1];
-        const int off = __float_as_int(tb.w);
-        const float4 r0 = P4[bi + off], r1 = P4[bi + dbi + off];
-        const float2 ex0 = f2add(f2lo(r0), nux0), ey0 = f2add(f2hi(r0), nuy0);
-        const float2 ex1 = f2add(f2lo(r1), nux1), ey1 = f2add(f2hi(r1), nuy1);
-        float2 dot0 = f2mul(ex0, f2lo(ta)), dot1 = f2mul(ex1, f2lo(ta));
-        dot0 = f2fma(ey0, f2hi(ta), dot0);
-        dot1 = f2fma(ey1, f2hi(ta), dot1);
-        float2 w0 = f2mul(dot0, f2lo(tb)), w1 = f2mul(dot1, f2lo(tb));
-        if (!LINEAR) {
-            const float2 ak = make_float2(tb.z, tb.z);
-            w0 = f2mul(w0, f2ex2(f2mul(ak, f2mul(dot0, dot0))));
-            w1 = f2mul(w1, f2ex2(f2mul(ak, f2mul(dot1, dot1))));
-        }
+    while (k < kend) {
+        const float4 *tw = tab + 2 * k;
+        const float4 first = tw[0];
+        const float2 dy = f2hi(first);
+        const int dx = (int)first.x, y = (int)first.z;
+        const int end = y == 0 && dx < 0 ? -1 : (int)__fsqrt_rn((float)(m * m - y * y));
+        int len = min(end - dx + 1, kend - k);
+        const int b0 = bi + __float_as_int(tw[1].w), odd = b0 & 1;
+        const float4 *A = P4 + (b0 >> 1) + (odd ? half : 0), *B = P4 + (b0 >> 1) + (odd ? 1 : half);
+        uint32_t m0 = 0, m1 = 0, m2 = 0, m3 = 0;
         if (MASKED) {
-            w0.x = ((c0 >> b) & 1u) ? w0.x : 0.f;
-            w0.y = ((c1 >> b) & 1u) ? w0.y : 0.f;
-            w1.x = ((c2 >> b) & 1u) ? w1.x : 0.f;
-            w1.y = ((c3 >> b) & 1u) ? w1.y : 0.f;
+            const int sh = k & 31;
+            m0 = c0 >> sh, m1 = c1 >> sh, m2 = c2 >> sh, m3 = c3 >> sh;
         }
-        Fx0 = f2fma(w0, f2lo(ta), Fx0);
-        Fy0 = f2fma(w0, f2hi(ta), Fy0);
-        Fx1 = f2fma(w1, f2lo(ta), Fx1);
-        Fy1 = f2fma(w1, f2hi(ta), Fy1);
+        k += len;
+        auto bond = [&](const float4 &r0, const float4 &r1, int b) {
+            const float2 dxx = reinterpret_cast<const float2 *>(tw + 2 * b)[0];
+            const float4 tb = tw[2 * b + 1];
+            const float2 ex0 = f2add(f2lo(r0), nux0), ey0 = f2add(f2hi(r0), nuy0);
+            const float2 ex1 = f2add(f2lo(r1), nux1), ey1 = f2add(f2hi(r1), nuy1);
+            float2 dot0 = f2mul(ex0, dxx), dot1 = f2mul(ex1, dxx);
+            dot0 = f2fma(ey0, dy, dot0);
+            dot1 = f2fma(ey1, dy, dot1);
+            float2 w0 = f2mul(dot0, f2lo(tb)), w1 = f2mul(dot1, f2lo(tb));
+            if (!LINEAR) {
+                const float2 ak = make_float2(tb.z, tb.z);
+                w0 = f2mul(w0, f2ex2(f2mul(ak, f2mul(dot0, dot0))));
+                w1 = f2mul(w1, f2ex2(f2mul(ak, f2mul(dot1, dot1))));
+            }
+            if (MASKED) {
+                w0.x = ((m0 >> b) & 1u) ? w0.x : 0.f;
+                w0.y = ((m1 >> b) & 1u) ? w0.y : 0.f;
+                w1.x = ((m2 >> b) & 1u) ? w1.x : 0.f;
+                w1.y = ((m3 >> b) & 1u) ? w1.y : 0.f;
+            }
+            Fx0 = f2fma(w0, dxx, Fx0);
+            Fy0 = f2fma(w0, dy, Fy0);
+            Fx1 = f2fma(w1, dxx, Fx1);
+            Fy1 = f2fma(w1, dy, Fy1);
+        };
+        float4 r = A[0];
+        auto run = [&](auto n) {       // n bonds (even)
+            constexpr int N = decltype(n)::value;
+#pragma unroll
+            for (int q = 0; q < N / 2; ++q) {
+                const float4 rb = B[q], ra = A[q + 1];
+                bond(r, rb, 2 * q);
+                bond(rb, ra, 2 * q + 1);
+                r = ra;
+            }
+            A += N / 2, B += N / 2, tw += 2 * N;
+            if (MASKED) m0 >>= N, m1 >>= N, m2 >>= N, m3 >>= N;
+        };
+#pragma unroll 1
+        for (; len >= PD_NP_ROW; len -= PD_NP_ROW) run(std::integral_constant<int, PD_NP_ROW>());
+#pragma unroll 1
+        for (; len >= 2; len -= 2) run(std::integral_constant<int, 2>());
+        if (len) bond(r, B[0], 0);
     }
 }
 
-// Launch: one CTA per tile, (tile points / 4) * a.split threads; thread (t, sub)
-// owns pairs t and t + T/4 and the sub-th of a.split ranges of stencil words.
+// Tiles a 2D tile's box reaches, in x and y, to either side.
+static __host__ __device__ inline int2 tile_reach(const Geom &g)
+{
+    return make_int2((g.m + g.bx - 1) >> g.lbx, (g.m + g.by - 1) >> g.lby);
+}
+constexpr int NP_LUT = 64;
+
+// Launch: one CTA per tile, (tile points / 4) * a.split threads; thread (t, sub) owns pairs
+// 2 t and 2 t + 1 and the sub-th of a.split ranges of stencil words.
 template <bool LINEAR>
-__global__ void __launch_bounds__(1024, 1) np_fast2(const TileArgs a)
+__global__ void __launch_bounds__(1024, 1) np_rows(const TileArgs a)
 {
     const Geom &g = a.g;
     const PairBox pb = pair_box(g);
-    const int S = g.S;
+    const int S = g.S, half = pb.n / 2;       // HX = bx + 2 m is even
     extern __shared__ float4 smem4[];
     float4 *P4 = smem4;
     float4 *tab = P4 + pb.n;                  // the layout of np_fast_smem in 2D
     constexpr int E = NP_TAB_WORDS(2);
-    __shared__ int s_nbr[27];
+    __shared__ int s_lut[NP_LUT];
     const int tile = blockIdx.x;
     const int4 org = __ldg(&a.tile_org[tile]);
-    for (int k = threadIdx.x; k < E * S; k += blockDim.x) tab[k] = __ldg(&a.tab_a[k]);
-    load_nbr(a, tile, s_nbr);
-    __syncthreads();
-    stage_pairs(a, pb, org, tile, s_nbr, P4, nullptr, false);
-    __syncthreads();
-
+    for (int k = threadIdx.x; k < E * S; k += blockDim.x)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(&tab[k])), "l"(&a.tab_a[k])
+                     : "memory");
+    const int2 reach = tile_reach(g);
+    const int ncx = 2 * reach.x + 1;
+    for (int k = threadIdx.x; k < ncx * (2 * reach.y + 1); k += blockDim.x) {
+        const int tx = (org.x >> g.lbx) - reach.x + k % ncx, ty = (org.y >> g.lby) - reach.y + k / ncx;
+        const bool in = tx >= 0 && ty >= 0 && (tx << g.lbx) < g.nx && (ty << g.lby) < g.ny;
+        s_lut[k] = in ? __ldg(&a.tile_lut[tx + g.tgx * ty]) : -1;
+    }
     const int npairs = g.T / 2, nthr = npairs / 2;     // nthr: a multiple of 32 (T >= 128)
     const int sub = threadIdx.x / nthr, t = threadIdx.x % nthr;
     const int w0 = sub * g.W / a.split, w1 = (sub + 1) * g.W / a.split;
-    const PairPts q0 = pair_points(g, pb, org, tile, t), q1 = pair_points(g, pb, org, tile, t + nthr);
-    const int dbi = q1.bi - q0.bi;
-    float2 Fx0, Fy0, Fx1, Fy1;
+    const PairPts q0 = pair_points(g, pb, org, tile, 2 * t), q1 = pair_points(g, pb, org, tile, 2 * t + 1);
+    // the words of the points x and x + 1 of a row stand side by side (nslots is even)
+    auto word = [&](int w, uint32_t *c) {
+        const size_t mo = (size_t)w * g.nslots;
+        const uint2 A = *reinterpret_cast<const uint2 *>(&a.mask[mo + q0.slot[0]]);
+        const uint2 B = *reinterpret_cast<const uint2 *>(&a.mask[mo + q0.slot[1]]);
+        c[0] = q0.act[0] ? A.x : 0u;
+        c[1] = q0.act[1] ? B.x : 0u;
+        c[2] = q1.act[0] ? A.y : 0u;
+        c[3] = q1.act[1] ? B.y : 0u;
+    };
+    auto full_word = [&](int w) { return S - 32 * w >= 32 ? 0xffffffffu : (1u << (S - 32 * w)) - 1u; };
+    // whether the warp has every bond of its range (read beside the staging's loads)
+    bool all = true;
+#pragma unroll 5
+    for (int w = w0; w < w1; ++w) {
+        uint32_t c[4];
+        word(w, c);
+        all = all && (c[0] & c[1] & c[2] & c[3]) == full_word(w);
+    }
+    all = __all_sync(0xffffffffu, all);
+    __syncthreads();
+    // Staging: every point of the box once (in a pair of rows each is both an A and a B),
+    // two rows side by side, so that a warp's loads share lines of the Morton order; the
+    // tiles from the table above (m may span several).
     {
-        const float4 u0 = P4[q0.bi], u1 = P4[q1.bi];
-        const float2 nux0 = f2neg(f2lo(u0)), nuy0 = f2neg(f2hi(u0));
-        const float2 nux1 = f2neg(f2lo(u1)), nuy1 = f2neg(f2hi(u1));
-        Fx0 = Fy0 = Fx1 = Fy1 = make_float2(0.f, 0.f);
-        const size_t mo0 = (size_t)w0 * g.nslots;
-        uint32_t n0 = q0.act[0] ? a.mask[mo0 + q0.slot[0]] : 0u;
-        uint32_t n1 = q0.act[1] ? a.mask[mo0 + q0.slot[1]] : 0u;
-        uint32_t n2 = q1.act[0] ? a.mask[mo0 + q1.slot[0]] : 0u;
-        uint32_t n3 = q1.act[1] ? a.mask[mo0 + q1.slot[1]] : 0u;
-        for (int w = w0; w < w1; ++w) {
-            const uint32_t m0 = n0, m1 = n1, m2 = n2, m3 = n3;
-            if (w + 1 < w1) {
-                const size_t mo = (size_t)(w + 1) * g.nslots;
-                n0 = q0.act[0] ? a.mask[mo + q0.slot[0]] : 0u;
-                n1 = q0.act[1] ? a.mask[mo + q0.slot[1]] : 0u;
-                n2 = q1.act[0] ? a.mask[mo + q1.slot[0]] : 0u;
-                n3 = q1.act[1] ? a.mask[mo + q1.slot[1]] : 0u;
+        const Ref32 ref = tile_ref32(a, tile);
+        const float inv_h = (float)a.inv_h, inv_row = __frcp_rn((float)(2 * pb.HX));
+        const int hb = g.by / 2;
+        float *P = reinterpret_cast<float *>(P4);
+#pragma unroll 4
+        for (int p = threadIdx.x; p < pb.HX * (pb.HY + hb); p += blockDim.x) {
+            const int r = fdiv_small(p, inv_row), rem = p - r * 2 * pb.HX, x = rem >> 1, y = 2 * r + (rem & 1);
+            const int gx = org.x - g.m + x, gy = org.y - g.m + y;
+            int s = -1;
+            if ((unsigned)gx < (unsigned)g.nx && (unsigned)gy < (unsigned)g.ny) {
+                const int tx = (gx >> g.lbx) - (org.x >> g.lbx) + reach.x, ty = (gy >> g.lby) - (org.y >> g.lby) + reach.y;
+                s = s_lut[tx + ncx * ty] * g.T + brick_code(2, gx & (g.bx - 1), gy & (g.by - 1), 0);
             }
-            const int nb = min(32, S - 32 * w);
-            const uint32_t full = nb == 32 ? 0xffffffffu : ((1u << nb) - 1u);
-            const float4 *tw = tab + E * 32 * w;
-            if (__all_sync(0xffffffffu, m0 == full && m1 == full && m2 == full && m3 == full))
-                np_word2<false, LINEAR>(tw, nb, P4, q0.bi, dbi, nux0, nuy0, nux1, nuy1, m0, m1, m2, m3, Fx0, Fy0,
-                                        Fx1, Fy1);
-            else
-                np_word2<true, LINEAR>(tw, nb, P4, q0.bi, dbi, nux0, nuy0, nux1, nuy1, m0, m1, m2, m3, Fx0, Fy0,
-                                       Fx1, Fy1);
+            const float4 v = stage_one(a, a.src_hl, s, ref, inv_h);
+            float *e = P + 4 * ((y * pb.HX + x) / 2 + (x & 1 ? half : 0));
+            if (y < pb.HY) e[0] = v.x, e[2] = v.y;
+            if (y >= hb) e -= 2 * hb * pb.HX, e[1] = v.x, e[3] = v.y;
         }
     }
-    float2 *red = reinterpret_cast<float2 *>(tab + E * S);
-    float2 Fz0 = make_float2(0.f, 0.f), Fz1 = Fz0;
-    if (a.split > 1) {
-        pair_split_sum(a, red, npairs, t, sub, Fx0, Fy0, Fz0);
-        pair_split_sum(a, red, npairs, t + nthr, sub, Fx1, Fy1, Fz1);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+
+    float2 Fx0, Fy0, Fx1, Fy1;
+    Fx0 = Fy0 = Fx1 = Fy1 = make_float2(0.f, 0.f);
+    {
+        const float4 u0 = P4[(q0.bi >> 1) + (q0.bi & 1 ? half : 0)], u1 = P4[(q1.bi >> 1) + (q1.bi & 1 ? half : 0)];
+        const float2 nux0 = f2neg(f2lo(u0)), nuy0 = f2neg(f2hi(u0));
+        const float2 nux1 = f2neg(f2lo(u1)), nuy1 = f2neg(f2hi(u1));
+        uint32_t nx[4] = {0u, 0u, 0u, 0u};
+        if (!all && w0 < w1) word(w0, nx);
+        for (int w = w0; w < w1;) {
+            const uint32_t c0 = nx[0], c1 = nx[1], c2 = nx[2], c3 = nx[3];
+            const int we = all ? w1 : w + 1;
+            if (we < w1) word(we, nx);
+            if (all || __all_sync(0xffffffffu, (c0 & c1 & c2 & c3) == full_word(w)))
+                np_row_bonds<false, LINEAR>(tab, g.m, 32 * w, min(S, 32 * we), P4, half, q0.bi, nux0, nuy0, nux1, nuy1,
+                                            0u, 0u, 0u, 0u, Fx0, Fy0, Fx1, Fy1);
+            else
+                np_row_bonds<true, LINEAR>(tab, g.m, 32 * w, min(S, 32 * we), P4, half, q0.bi, nux0, nuy0, nux1, nuy1,
+                                           c0, c1, c2, c3, Fx0, Fy0, Fx1, Fy1);
+            w = we;
+        }
     }
-    if (sub == 0) {
-        const float FA0[3] = {Fx0.x, Fy0.x, 0.f}, FB0[3] = {Fx0.y, Fy0.y, 0.f};
-        pair_epilogue2(a, q0, FA0, FB0, 2);
-        const float FA1[3] = {Fx1.x, Fy1.x, 0.f}, FB1[3] = {Fx1.y, Fy1.y, 0.f};
-        pair_epilogue2(a, q1, FA1, FB1, 2);
+    // The ranges' sums in order, and the update, over all of the threads: with 4 ranges a
+    // point each. The box is done with and holds the sums.
+    float4 *red = P4;                         // [range][pair] {Fx, Fy}: launch_np_fast checks that it fits
+    if (a.split > 1) {
+        __syncthreads();
+        red[sub * npairs + 2 * t] = make_float4(Fx0.x, Fx0.y, Fy0.x, Fy0.y);
+        red[sub * npairs + 2 * t + 1] = make_float4(Fx1.x, Fx1.y, Fy1.x, Fy1.y);
+        __syncthreads();
+    }
+    for (int i = a.split > 1 ? sub & 1 : 0; i < 2; i += a.split > 1 ? 2 : 1) {
+        PairPts q = pair_points(g, pb, org, tile, 2 * t + i);
+        if (a.split == 4) q.act[1 - sub / 2] = false;
+        float2 Fx = i ? Fx1 : Fx0, Fy = i ? Fy1 : Fy0;
+        if (a.split > 1) {
+            float4 r = red[2 * t + i];
+            Fx = f2lo(r), Fy = f2hi(r);
+            for (int j = 1; j < a.split; ++j) {
+                r = red[j * npairs + 2 * t + i];
+                Fx = f2add(Fx, f2lo(r));
+                Fy = f2add(Fy, f2hi(r));
+            }
+        }
+        const float FA[3] = {Fx.x, Fy.x, 0.f}, FB[3] = {Fx.y, Fy.y, 0.f};
+        pair_epilogue2(a, q, FA, FB, 2);
     }
 }
 
@@ -359,11 +467,11 @@ static int launch_np_split(const TileArgs &a, cudaStream_t st)
 }
 
 template <bool LINEAR>
-static int launch_np_fast2(const TileArgs &a, cudaStream_t st)
+static int launch_np_rows(const TileArgs &a, cudaStream_t st)
 {
-    const size_t smem = split_smem(a.g, np_fast_smem(a.g), a.split);
-    PD_CUDA(smem_limit(np_fast2<LINEAR>, smem));
-    np_fast2<LINEAR><<<a.g.ntiles, a.g.T / 4 * a.split, smem, st>>>(a);
+    const size_t smem = np_fast_smem(a.g);
+    PD_CUDA(smem_limit(np_rows<LINEAR>, smem));
+    np_rows<LINEAR><<<a.g.ntiles, a.g.T / 4 * a.split, smem, st>>>(a);
     PD_CUDA(cudaGetLastError());
     return PD_OK;
 }
@@ -373,10 +481,15 @@ static int launch_np_fast(const TileArgs &a0, cudaStream_t st)
 {
     TileArgs a = a0;   // pair_threads applies to PMB only: the split is chosen here
     a.split = choose_split(a.g, np_fast_smem(a.g));
-    // 2D wide horizons (the one-pair kernel would split): two pairs per thread
+    // 2D wide horizons (the one-pair kernel would split): two pairs per thread by rows
     if (DIM == 2 && a.split > 1 && a.g.T >= 128) {
-        a.split = choose_split(a.g, np_fast_smem(a.g), 2);
-        return launch_np_fast2<LINEAR>(a, st);
+        const int split = choose_split(a.g, np_fast_smem(a.g), 2);
+        const int2 r = tile_reach(a.g);
+        const int box = (a.g.bx + 2 * a.g.m) * (a.g.by / 2 + 2 * a.g.m);
+        if ((2 * r.x + 1) * (2 * r.y + 1) <= NP_LUT && split * a.g.T / 2 <= box) {
+            a.split = split;
+            return launch_np_rows<LINEAR>(a, st);
+        }
     }
     return a.split > 1 ? launch_np_split<DIM, LINEAR, true>(a, st) : launch_np_split<DIM, LINEAR, false>(a, st);
 }
