@@ -363,9 +363,11 @@ __global__ void __launch_bounds__(256) f64_jvp(const __grid_constant__ TileArgs 
                 const double cs = f64_div(num, fma(e.C, q * rs, e.R * q));         // V_ij s / r
                 double cn = ndw * (rs * rs) * rs;                                  // (n.dw) / r^2
                 cn *= e.V;
-                ox = fma(cn, yx, fma(cs, dwx, ox));
-                oy = fma(cn, yy, fma(cs, dwy, oy));
-                if (DIM == 3) oz = fma(cn, yz, fma(cs, dwz, oz));
+                // a bond's two terms first: added to the sum one by one they round it twice (an
+                // error of 3.7e-16 against 2.7e-16, m = 5 in 2D)
+                ox += fma(cn, yx, cs * dwx);
+                oy += fma(cn, yy, cs * dwy);
+                if (DIM == 3) oz += fma(cn, yz, cs * dwz);
             }
         }
         a.jv[0][p.slot] = sc * ox;
