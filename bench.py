@@ -60,7 +60,8 @@ ALG_BYTES = {"pmb3": (4.25, 110.0), "pmb2": (4.25, 76.0), "lps_dil": (4.0, 44.0)
 # 2D NP at m = 20: the same with 40 mask words (290).
 PER_POINT_BYTES = {"pmb3": 179.0, "pmb2": 134.0, "lps_dil": 56.0, "lps_force": 187.0, "np2": 290.0}
 PASS_KERNEL = {"pmb3": "pmb_fast<3, *> (fused force + update)", "pmb2": "pmb_fast<2, *> (fused force + update)",
-               "lps_dil": "lps_dil_fast2 (dilatation pass)", "lps_force": "lps_force_fast (force + update pass)",
+               "lps_dil": "rows (dilatation pass by stencil rows; lps_dil_fast2 on small grids)",
+               "lps_force": "rows (force + update pass by stencil rows; lps_force_fast on small grids)",
                "np2": "np_rows (fused force + update, two point pairs per thread by stencil rows)"}
 FALLBACK_HBM_GBS = 6800.0
 
@@ -70,12 +71,13 @@ FALLBACK_HBM_GBS = 6800.0
 # flags hash to the value recorded with it; otherwise traffic is null.
 _KERNEL_COMMON = ["paper_1806_06917_gb300/csrc/pd_internal.cuh", "paper_1806_06917_gb300/csrc/pd_tile.cuh",
                   "paper_1806_06917_gb300/csrc/pd_pair.cuh", "paper_1806_06917_gb300/build.py"]
-_LPS_SOURCES = ["paper_1806_06917_gb300/csrc/pd_force_lps.cu", "paper_1806_06917_gb300/csrc/pd_lps_fast.cuh"]
+_LPS_SOURCES = ["paper_1806_06917_gb300/csrc/pd_force_lps.cu", "paper_1806_06917_gb300/csrc/pd_lps_fast.cuh",
+                "paper_1806_06917_gb300/csrc/pd_rows.cu", "paper_1806_06917_gb300/csrc/pd_rows.cuh"]
 NCU_TRAFFIC = {
     # (pass key, tile_log2): the capture of that kernel at that tile size
-    ("lps_dil", 9): {"bytes": 109745408 + 6098176, "sha": "e7864e5b1918a9c7",
+    ("lps_dil", 9): {"bytes": 110454016 + 6153216, "sha": "dd9acf0d41ba2ca5",
                      "sources": _LPS_SOURCES + _KERNEL_COMMON, "profile": "profiles/lps_block3d_128.md"},
-    ("lps_force", 9): {"bytes": 230127872 + 123059968, "sha": "e7864e5b1918a9c7",
+    ("lps_force", 9): {"bytes": 231078656 + 123772416, "sha": "dd9acf0d41ba2ca5",
                        "sources": _LPS_SOURCES + _KERNEL_COMMON, "profile": "profiles/lps_block3d_128.md"},
 }
 
