@@ -19,7 +19,7 @@
 // third-order steps leave an error of the order of the last rounding. 64^3 PMB step with
 // breaking 3.58 -> 1.64 ms (27 instructions a bond cost 1.40), 40^3 LPS step 1.70 -> 0.90 ms, 97^2
 // NP step (m = 8; its exponential by a short series near 0) 2.06 -> 0.165 ms, tangent product
-// and force of the 200^2 plate through the torch bridge 0.556 -> 0.242 ms. The error against 64-bit
+// and force of the 200^2 plate through the torch bridge 0.556 -> 0.251 ms. The error against 64-bit
 // references stays at the last bits (2 to 5e-16).
 #include <algorithm>
 
