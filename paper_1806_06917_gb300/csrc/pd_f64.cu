@@ -15,7 +15,7 @@
 //         one quotient, from rcp.approx.ftz.f64 and a third-order step
 //         (g = 1 - den y0, num y0 (1 + g + g^2))                              2 + 4
 //   F  += w y                                                                 3 + 3
-// 27 in 3D and 21 in 2D (dilatation 21, LPS force 32, tangent product 40 and 29). Both
+// 27 in 3D and 21 in 2D (dilatation 21, LPS force 32, tangent product 43 and 31). Both
 // third-order steps leave an error of the order of the last rounding. 64^3 PMB step with
 // breaking 3.58 -> 1.64 ms (27 instructions a bond cost 1.40), 40^3 LPS step 1.70 -> 0.90 ms, 97^2
 // NP step (m = 8; its exponential by a short series near 0) 2.06 -> 0.165 ms, tangent product
