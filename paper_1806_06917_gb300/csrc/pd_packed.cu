@@ -106,8 +106,8 @@ static __device__ __forceinline__ void pk_lps_force(const TileArgs &a, int tile,
 {
     lps_force_fast_body<false, true>(a, tile, tab);
 }
-static __device__ __forceinline__ void pk_pmb3s(const TileArgs &a, int tile) { pmb_fast_body<3, false, true, false>(a, tile, nullptr); }
-static __device__ __forceinline__ void pk_pmb3(const TileArgs &a, int tile) { pmb_fast_body<3, false, false, false>(a, tile, nullptr); }
+static __device__ __forceinline__ void pk_pmb3s(const TileArgs &a, int tile) { pmb_fast_body<3, false, true, false, false>(a, tile, nullptr); }
+static __device__ __forceinline__ void pk_pmb3(const TileArgs &a, int tile) { pmb_fast_body<3, false, false, false, false>(a, tile, nullptr); }
 static __device__ __forceinline__ void pk_pmb2s(const TileArgs &a, int tile) { pmb_fast_body<2, false, true, false>(a, tile, nullptr); }
 static __device__ __forceinline__ void pk_pmb2(const TileArgs &a, int tile) { pmb_fast_body<2, false, false, false>(a, tile, nullptr); }
 

@@ -244,7 +244,11 @@ __device__ __forceinline__ void pair_split_sum(const TileArgs &a, float2 *red, i
 // blockIdx.x; the request server's packed kernel (pd_packed.cu) runs it for the
 // tiles of its work items, with a in shared memory.
 // PTAB: the table is read from ptab (a kernel parameter) instead of shared memory.
-template <int DIM, bool BRK, bool SPLIT, bool PTAB>
+// COLS: grids of many or ragged tiles are staged by columns (stage_pairs). The packed
+// kernel leaves that out: beside its other bodies in 64 registers it spilled 496 bytes a
+// thread instead of 196, which every request paid for (128^3 LPS alone 0.573 -> 0.617 ms a
+// step, twelve mixed requests 15.5 -> 16.2 ms).
+template <int DIM, bool BRK, bool SPLIT, bool PTAB, bool COLS = DIM == 3 && !PTAB>
 __device__ __forceinline__ void pmb_fast_body(const TileArgs &a, int tile, const float4 *ptab)
 {
     const Geom &g = a.g;
@@ -288,7 +292,7 @@ __device__ __forceinline__ void pmb_fast_body(const TileArgs &a, int tile, const
     }
     load_nbr(a, tile, s_nbr);
     __syncthreads();
-    stage_pairs<DIM == 3 && !PTAB>(a, pb, org, tile, s_nbr, P4, DIM == 3 ? P2 : nullptr, true);
+    stage_pairs<COLS>(a, pb, org, tile, s_nbr, P4, DIM == 3 ? P2 : nullptr, true);
     if (tab2) {
         if (k0 < 4 * S) tab[k0] = t0;
         if (k1 < 4 * S) tab[k1] = t1;
