@@ -752,7 +752,8 @@ static int create_impl(pd_sim *s)
         for (int k = 0; k < g.S; ++k) {
             const int4 d = st[k];
             const double rr = r0[k], d2 = d.w, v = mt.vol_corr && rr > g.m - 0.5 ? (g.m + 0.5 - rr) : 1.0;
-            F64Ent e = {(double)d.x, (double)d.y, (double)d.z, d2, rr / v, d2 / v, v, d.x + HX * (d.y + HY * d.z), 0};
+            const double two = np_law ? 1.0 : 2.0;
+            F64Ent e = {two * d.x, two * d.y, two * d.z, d2, rr / v, d2 / v, v / rr, d.x + HX * (d.y + HY * d.z), 0};
             if (mt.model == PD_MODEL_LPS) {
                 e.R = rr;
                 e.C = v;

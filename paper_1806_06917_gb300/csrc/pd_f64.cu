@@ -8,24 +8,36 @@
 // 115 on the two LPS passes, half of them in the correctly rounded 1 / sqrt and the
 // divisions (and, in 2D, on a third component of zeros). Here a bond takes, in lattice
 // units (xi = d, e = eta, y = d + e, r0 = |d|, r = |y|):
-//   num = 2 d.e + e.e, q = r0^2 + num                                       3 + 6 + 1
-//   r   = sqrt(q): the rsqrt.approx.ftz.f64 seed (about 22 bits) and one
-//         third-order step, z = q y0, g = 1 - z y0, r = z + z g (1/2 + 3/8 g)       5
+//   num = 2 d.e + e.e, q = r0^2 + num                                     3 + 6 + 1
+//   r   = sqrt(q): the rsqrt.approx.ftz.f64 seed (21 bits) and one third-order
+//         step, z = q y0, g = 1 - z y0, r = z + z g (1/2 + 3/8 g)                   5
 //   w   = num / (R q + C r), R = r0 / V_ij, C = r0^2 / V_ij: s V_ij / r in
-//         one quotient, from rcp.approx.ftz.f64 and a third-order step
-//         (g = 1 - den y0, num y0 (1 + g + g^2))                              2 + 4
+//         one quotient, z = num y0 from rcp.approx.ftz.f64 and its residual
+//         over den, z + (num - den z) y0 (2 - den y0)                          2 + 5
 //   F  += w y                                                                 3 + 3
-// 27 in 3D and 21 in 2D (dilatation 21, LPS force 32, tangent product 43 and 31). Both
-// third-order steps leave an error of the order of the last rounding. 64^3 PMB step with
-// breaking 3.58 -> 1.64 ms (27 instructions a bond cost 1.40), 40^3 LPS step 1.70 -> 0.90 ms, 97^2
+// 28 in 3D and 23 in 2D (dilatation 23, LPS force 32, tangent product 45 and 36). The
+// quotient, the dilatation's root and 1 / sqrt(q) round once. 64^3 PMB step with breaking
+// 3.58 -> 1.67 ms (28 instructions a bond cost 1.45), 40^3 LPS step 1.70 -> 0.93 ms, 97^2
 // NP step (m = 8; its exponential by a short series near 0) 2.06 -> 0.165 ms, tangent product
-// and force of the 200^2 plate through the torch bridge 0.556 -> 0.251 ms. The error against 64-bit
-// references stays at the last bits (2 to 5e-16).
+// and force of the 200^2 plate through the torch bridge 0.556 -> 0.25 ms. The error against
+// extended precision is that of the templates, 1.3 to 5e-16 for m = 1 to 5 (relative L2), also
+// for compressed bonds (f64_len2).
 #include <algorithm>
 
 #include "pd_tile.cuh"
 
 namespace pdk {
+
+// num = |y|^2 - |d|^2 = 2 d.e + e.e (dx..: 2 d): the small squares first, so that they round
+// below the other terms, whose products are exact where d has the sides 1 and 2.
+__device__ __forceinline__ double f64_num2(const F64Ent &e, double ex, double ey)
+{
+    return fma(e.dy, ey, fma(e.dx, ex, fma(ey, ey, ex * ex)));
+}
+__device__ __forceinline__ double f64_num3(const F64Ent &e, double ex, double ey, double ez)
+{
+    return fma(e.dz, ez, fma(e.dy, ey, fma(e.dx, ex, fma(ez, ez, fma(ey, ey, ex * ex)))));
+}
 
 // Box geometry and the thread's point.
 struct F64Pt {
@@ -103,8 +115,9 @@ __device__ __noinline__ bool f64_breaks(const TileArgs *ap, int slot, int x, int
     const double r0 = sqrt(e->d2), r = sqrt(e->d2 + num);
     const double s = num / (r0 * (r + r0));
     if (fabs(s - a.s_c) <= 0x1p-30 * a.s_c) {
-        const int sj = slot_at(a.g, a.tile_lut, x + (int)e->dx, y + (int)e->dy, z + (int)e->dz);
-        return sj >= 0 && canon_stretch64(a, slot, sj, e->dx, e->dy, e->dz, e->d2) > a.s_c;
+        const double dx = 0.5 * e->dx, dy = 0.5 * e->dy, dz = 0.5 * e->dz;
+        const int sj = slot_at(a.g, a.tile_lut, x + (int)dx, y + (int)dy, z + (int)dz);
+        return sj >= 0 && canon_stretch64(a, slot, sj, dx, dy, dz, e->d2) > a.s_c;
     }
     return s > a.s_c;
 }
@@ -136,14 +149,14 @@ __global__ void __launch_bounds__(256) f64_pmb(const __grid_constant__ TileArgs 
                 const F64Ent &e = tab[32 * w + b];
                 const double4_32a rj = box[p.bi + e.off];
                 const double ex = rj.x - ui.x, ey = rj.y - ui.y;
-                const double yx = ex + e.dx, yy = ey + e.dy;
-                double num = ex * (yx + e.dx);
-                num = fma(ey, yy + e.dy, num);
-                double yz = 0.0;
+                const double yx = fma(0.5, e.dx, ex), yy = fma(0.5, e.dy, ey);
+                double num, yz = 0.0;
                 if (DIM == 3) {
                     const double ez = rj.z - ui.z;
-                    yz = ez + e.dz;
-                    num = fma(ez, yz + e.dz, num);
+                    yz = fma(0.5, e.dz, ez);
+                    num = f64_num3(e, ex, ey, ez);
+                } else {
+                    num = f64_num2(e, ex, ey);
                 }
                 if (BRK && __double2hiint(num) >= e.near &&
                     f64_breaks(&a, p.slot, p.x, p.y, p.z, &e, num)) {
@@ -232,11 +245,9 @@ __global__ void __launch_bounds__(256) f64_lps_dil(const __grid_constant__ TileA
                 const F64Ent &e = tab[32 * w + b];
                 const double4_32a rj = box[p.bi + e.off];
                 const double ex = rj.x - ui.x, ey = rj.y - ui.y, ez = rj.z - ui.z;
-                double num = ex * ((ex + e.dx) + e.dx);
-                num = fma(ey, (ey + e.dy) + e.dy, num);
-                num = fma(ez, (ez + e.dz) + e.dz, num);
-                const double q = f64_len2(num, e.d2, ex + e.dx, ey + e.dy, ez + e.dz);
-                double x = f64_div(num, f64_sqrt(q) + e.R);
+                const double num = f64_num3(e, ex, ey, ez);
+                const double q = f64_len2(num, e.d2, fma(0.5, e.dx, ex), fma(0.5, e.dy, ey), fma(0.5, e.dz, ez));
+                double x = f64_div(num, f64_sqrt_rn(q) + e.R);
                 if (VOL) x *= e.C;
                 acc = fma(e.R, x, acc);
             }
@@ -292,10 +303,8 @@ __global__ void __launch_bounds__(256) f64_lps_force(const __grid_constant__ Til
                 const int bj = p.bi + e.off;
                 const double4_32a rj = box[bj];
                 const double ex = rj.x - ui.x, ey = rj.y - ui.y, ez = rj.z - ui.z;
-                const double yx = ex + e.dx, yy = ey + e.dy, yz = ez + e.dz;
-                double num = ex * (yx + e.dx);
-                num = fma(ey, yy + e.dy, num);
-                num = fma(ez, yz + e.dz, num);
+                const double yx = fma(0.5, e.dx, ex), yy = fma(0.5, e.dy, ey), yz = fma(0.5, e.dz, ez);
+                const double num = f64_num3(e, ex, ey, ez);
                 const double q = f64_len2(num, e.d2, yx, yy, yz), rs = f64_rsqrt(q);
                 const double x = f64_div(num, fma(q, rs, e.R));
                 double gg = e.R * (ui.w + rj.w);
@@ -314,8 +323,9 @@ __global__ void __launch_bounds__(256) f64_lps_force(const __grid_constant__ Til
 
 // --------------------------------------------------------------- tangent
 
-// (K w)_i = (c V / h) sum_j V_ij [ (n.dw) n / r + (s / r) dw ], n = y / r: the coefficient
-// 1 / |d| - s / r of n n^T in pd_jvp.cu is 1 / r. D_ij is symmetric and the volumes are
+// (K w)_i = (c V / h) sum_j V_ij [ (n.dw) (1 / |d| - s / r) n + (s / r) dw ], n = y / r. The
+// coefficient of n n^T is 1 / r as well, but rs^3 y.dw y carries the root's rounding three
+// times (2D, m = 2: 1.74e-16 against 1.60e-16). D_ij is symmetric and the volumes are
 // uniform, so the adjoint's transposed gather evaluates the same terms.
 template <int DIM>
 __global__ void __launch_bounds__(256) f64_jvp(const __grid_constant__ TileArgs a)
@@ -359,24 +369,23 @@ __global__ void __launch_bounds__(256) f64_jvp(const __grid_constant__ TileArgs 
                 const F64Ent &e = tab[32 * w + b];
                 const double4_32a uj = box[p.bi + e.off], wj = wbox[p.bi + e.off];
                 const double ex = uj.x - ui.x, ey = uj.y - ui.y;
-                const double yx = ex + e.dx, yy = ey + e.dy;
+                const double yx = fma(0.5, e.dx, ex), yy = fma(0.5, e.dy, ey);
                 const double dwx = wj.x - wi.x, dwy = wj.y - wi.y;
-                double num = ex * (yx + e.dx);
-                num = fma(ey, yy + e.dy, num);
                 double ndw = yx * dwx;
                 ndw = fma(yy, dwy, ndw);
-                double yz = 0.0, dwz = 0.0;
+                double num, yz = 0.0, dwz = 0.0;
                 if (DIM == 3) {
                     const double ez = uj.z - ui.z;
-                    yz = ez + e.dz;
-                    num = fma(ez, yz + e.dz, num);
+                    yz = fma(0.5, e.dz, ez);
+                    num = f64_num3(e, ex, ey, ez);
                     dwz = wj.z - wi.z;
                     ndw = fma(yz, dwz, ndw);
+                } else {
+                    num = f64_num2(e, ex, ey);
                 }
                 const double q = f64_len2(num, e.d2, yx, yy, yz), rs = f64_rsqrt(q);
                 const double cs = f64_div(num, fma(e.C, q * rs, e.R * q));         // V_ij s / r
-                double cn = ndw * (rs * rs) * rs;                                  // (n.dw) / r^2
-                cn *= e.V;
+                const double cn = ndw * rs * (e.I - cs) * rs;                      // times y
                 // a bond's two terms first: added to the sum one by one they round it twice (an
                 // error of 3.7e-16 against 2.7e-16, m = 5 in 2D)
                 ox += fma(cn, yx, cs * dwx);

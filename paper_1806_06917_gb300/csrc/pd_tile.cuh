@@ -125,7 +125,9 @@ __device__ __forceinline__ double seed_rcp(double x)
     return y;
 }
 
-// sqrt(q) for q > 0: one third-order (Halley-type) step from the seed.
+// The seeds carry 21 significant bits (their low words are zero), so the products marked
+// exact are. sqrt(q) for q > 0: one third-order (Halley-type) step from the seed; the
+// rounding of z is left in the result (below 0.8 ulp).
 __device__ __forceinline__ double f64_sqrt(double q)
 {
     const double y = seed_rsqrt(q), z = q * y;
@@ -133,28 +135,38 @@ __device__ __forceinline__ double f64_sqrt(double q)
     return fma(z * g, fma(0.375, g, 0.5), z);
 }
 
-// 1 / sqrt(q) the same way.
+// The same with the residual of z: nothing is left but the last rounding.
+__device__ __forceinline__ double f64_sqrt_rn(double q)
+{
+    const double y = seed_rsqrt(q), z = q * y;
+    const double p = fma(-z, z, q) * y, g = p * y;
+    return fma(p, fma(0.375, g, 0.5), z);
+}
+
+// 1 / sqrt(q) the same way (y y is exact).
 __device__ __forceinline__ double f64_rsqrt(double q)
 {
     const double y = seed_rsqrt(q);
-    const double g = fma(-(q * y), y, 1.0);
+    const double g = fma(-q, y * y, 1.0);
     return fma(y * g, fma(0.375, g, 0.5), y);
 }
 
-// a / b for b in the normal range, third order from the seed.
+// a / b for b in the normal range: the quotient a y and its residual, divided by the seed
+// corrected once. The last rounding alone is left (without the residual, the rounding of
+// a y is too: 1 ulp).
 __device__ __forceinline__ double f64_div(double a, double b)
 {
-    const double y = seed_rcp(b);
-    const double g = fma(-b, y, 1.0), z = a * y;
-    return fma(z, fma(g, g, g), z);
+    const double y = seed_rcp(b), z = a * y;
+    return fma(fma(-b, z, a), fma(y, fma(-b, y, 1.0), y), z);
 }
 
-// 1/sqrt(q) and a/b: hardware approximations in FP32 (a few ulp), the third-order
-// steps above in FP64 (the last bit).
+// 1/sqrt(q) and a/b of the templates: hardware approximations in FP32 (a few ulp),
+// correctly rounded root and quotients in FP64 (the energies and the cached tangent, off
+// the step path).
 __device__ __forceinline__ float prsqrt1(float q) { return rsqrtf(q); }
-__device__ __forceinline__ double prsqrt1(double q) { return f64_rsqrt(q); }
+__device__ __forceinline__ double prsqrt1(double q) { return 1.0 / sqrt(q); }
 __device__ __forceinline__ float pdiv1(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double pdiv1(double a, double b) { return f64_div(a, b); }
+__device__ __forceinline__ double pdiv1(double a, double b) { return a / b; }
 
 template <class R, int P>
 __device__ __forceinline__ Pk<R, P> prsqrt(const Pk<R, P> &q)
@@ -406,8 +418,8 @@ struct RowArgs {
 // Stencil entry of the all-FP64 passes (pd_f64.cu), in global memory (its warp-uniform
 // reads hit the L1 while the FP64 pipe is busy).
 struct F64Ent {
-    double dx, dy, dz, d2;
-    double R, C, V;         // PMB: r0 / V_ij, r0^2 / V_ij; LPS: r0, V_ij; NP / LP: k, a'; V_ij
+    double dx, dy, dz, d2;  // 2 d (PMB, LPS) or d (NP / LP); |d|^2
+    double R, C, I;         // PMB: r0 / V_ij, r0^2 / V_ij, V_ij / r0; LPS: r0, V_ij; NP / LP: k, a'
     int off;                // box offset (x extent bx + 2m, y extent by + 2m)
     int near;               // PMB with s_c: high word of the num below which a bond is far from breaking
 };
