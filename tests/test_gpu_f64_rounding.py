@@ -64,3 +64,22 @@ def test_energy_divides_and_takes_roots_in_ieee_arithmetic(pd):
         s = (q - 1.0) / den
         want.append(k * (s * s))
     assert any((got == w).all() for w in want), [int((got != w).sum()) for w in want]
+
+
+@pytest.mark.parametrize("model", [W.NP, W.LP])
+def test_points_at_the_horizon_do_not_act(pd, model):
+    """J = 0 at |xi| = delta (NP, LP): a displacement without bound there leaves the force
+    alone. (5, 5) is no tile's reference point; those at a distance below 3 do see it."""
+    g = W.Grid(dim=2, n=(17, 15, 1), h=0.25, m=3)
+    sim = pd.pd_create(*pd.describe(g, W.Material(model=model, rho=1.0, psi_c=1.0, psi_beta=1.0),
+                                    precision=pd.PD_FP64, dt=1e-5))
+    pd.pd_build_neighbors(sim)
+    u = W.random_field(g, 0.01 * g.h, seed=2)
+    f0 = pd.pd_force(sim, u=u)
+    c = g.coords()[:, :2]
+    r2 = ((c - [5, 5]) ** 2).sum(1)
+    u[r2 == 0] = np.inf
+    f = pd.pd_force(sim, u=u)
+    sim.close()
+    assert (r2 == 9).sum() == 4
+    assert (f[r2 >= 9] == f0[r2 >= 9]).all()
