@@ -759,6 +759,8 @@ static int create_impl(pd_sim *s)
                 e.C = v;
             } else if (np_law) {    // S / |d| = p / (d2 |d|), exponent -beta h |d| S^2 = a' p^2, p = d.e; J = 0 at m
                 e.R = d2 < (double)g.m * g.m ? v / (rr * d2) : 0.0;
+                // at the horizon the own point stands in, so that a neighbour at infinity does not act
+                if (e.R == 0.0) e.off = 0;
                 e.C = -mt.psi_beta * g.h * rr / (d2 * d2);
             }
             const double near = d2 * mt.s_c * (2.0 + mt.s_c) * (1.0 - 0x1p-16);

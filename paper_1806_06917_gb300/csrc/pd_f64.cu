@@ -199,9 +199,8 @@ __global__ void __launch_bounds__(256) f64_np(const __grid_constant__ TileArgs a
             const int nb = min(32, g.S - 32 * w);
 #pragma unroll 4
             for (int b = 0; b < nb; ++b) {
+                if (!((word >> b) & 1u)) continue;
                 const F64Ent &e = tab[32 * w + b];
-                // (J = 0 at the horizon, where k = 0: no bond, also to a point at infinity)
-                if (!((word >> b) & 1u) || __double2hiint(e.R) == 0) continue;
                 const double4_32a rj = box[p.bi + e.off];
                 double dot = (rj.x - ui.x) * e.dx;
                 dot = fma(rj.y - ui.y, e.dy, dot);
