@@ -487,7 +487,7 @@ static int create_impl(pd_sim *s)
     // adds 1-3 % (64^3 PMB step: 1.84 ms with 512 tiles of 2^9, 1.65 with 1024 of 2^8; 40^3 LPS: 1.01
     // with 125 tiles of 2^9, 0.90 with 1000 of 2^6)
     if (s->precision == PD_FP64 && !s->run.tile_log2)
-        for (int L = g.L; L > 6 && (long long)g.tgx * g.tgy * g.tgz < 6 * 152;) set_tile(--L);
+        for (int L = g.L; L > 6 && (long long)g.tgx * g.tgy * g.tgz < 6 * SMS;) set_tile(--L);
     s->tangent_ok = tangent;
 
     // tiles: bricks intersecting the grid, ordered by the Morton code of their origin
@@ -771,7 +771,8 @@ static int create_impl(pd_sim *s)
         }
         s->plan.filled(s->tab64, tab);
     }
-    if (s->precision == PD_FP32C && g.dim == 3 && g.L == 9 && s->nbr_ok && !np_law) {
+    if (s->precision == PD_FP32C && g.dim == 3 && g.L == 9 && s->nbr_ok &&
+        (mt.model == PD_MODEL_LPS || (!np_law && rows_pmb(g)))) {
         const int rc = create_rows(s, st);
         if (rc != PD_OK) return rc;
     }

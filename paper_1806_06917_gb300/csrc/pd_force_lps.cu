@@ -17,6 +17,7 @@
 namespace pdk {
 
 int launch_rows_lps(const TileArgs &a, const RowArgs &ra, int dil, cudaStream_t st);
+size_t rows_smem(const RowArgs &ra, bool force, bool param_table);
 int launch_f64_lps(const TileArgs &a, int dil, size_t smem, cudaStream_t st);
 
 size_t lps_fast_smem(const Geom &g, bool dil)
@@ -41,7 +42,7 @@ int launch_lps_args(const TileArgs &a, int precision, int dil, cudaStream_t st)
 {
     const Geom &g = a.g;
     const size_t smem = lps_generic_smem(g, precision, dil);
-    if (precision == PD_FP32C && a.rows && g.ntiles >= (dil ? ROWS_MIN_TILES : ROWS_MIN_TILES_FRC))
+    if (precision == PD_FP32C && a.rows && (dil ? rows_dil(g) : rows_frc(g, rows_smem(a.rows[1], true, false))))
         return launch_rows_lps(a, a.rows[dil ? 0 : 1], dil, st);
     if (precision == PD_FP32C) {
         // dilatation: two pairs per thread from 2^7-point tiles and two stencil words on
@@ -53,7 +54,7 @@ int launch_lps_args(const TileArgs &a, int precision, int dil, cudaStream_t st)
         // (the dilatation's table is tab_a, the force pass's tab_b)
         const float4 *ht = dil ? a.htab_a : a.htab_b;
         const int nt = dil ? a.ntab_a : a.ntab_b;
-        const bool pt = ht && nt > 0 && nt <= PTAB_N && g.ntiles >= 2048;
+        const bool pt = ht && nt > 0 && nt <= PTAB_N && g.ntiles >= PTAB_MIN_TILES;
         if (pt) {
             memcpy(tp.e, ht, sizeof(float4) * (size_t)nt);
             auto k = dil ? (dil2 ? (a.vol_corr ? lps_dil_fast2_pt<true> : lps_dil_fast2_pt<false>)
@@ -62,7 +63,9 @@ int launch_lps_args(const TileArgs &a, int precision, int dil, cudaStream_t st)
             PD_CUDA(smem_limit(k, smem));
             k<<<g.ntiles, threads, smem, st>>>(a, tp);
         } else {
-            auto k = dil ? (dil2 ? (a.vol_corr ? lps_dil_fast2<true> : lps_dil_fast2<false>)
+            const bool cols = cols_staging(a) && (g.ntiles >= ROWS_MIN_TILES || ragged(a));
+            auto k = dil ? (dil2 ? (cols ? (a.vol_corr ? lps_dil_fast2<true, true> : lps_dil_fast2<false, true>)
+                                         : (a.vol_corr ? lps_dil_fast2<true, false> : lps_dil_fast2<false, false>))
                                  : (a.vol_corr ? lps_dil_fast<true> : lps_dil_fast<false>))
                          : (a.vol_corr ? lps_force_fast<true> : lps_force_fast<false>);
             PD_CUDA(smem_limit(k, smem));

@@ -406,13 +406,34 @@ int pmb_split(const Geom &g, int pair_threads)
 // shared-memory pipe that the table's reads would share (256^3 PMB step 2.43 ->
 // 2.33 ms), while a grid of about one wave, bound by latency, measured slower
 // with it (64^3: 0.064 -> 0.069 ms).
-constexpr int PTAB_MIN_TILES = 2048;
-
 static bool param_table(const float4 *host, int n, int ntiles, ParamTab &tp)
 {
     if (!host || n <= 0 || n > PTAB_N || ntiles < PTAB_MIN_TILES) return false;
     memcpy(tp.e, host, sizeof(float4) * (size_t)n);
     return true;
+}
+
+// Staging by columns (us a step, by pairs and by columns). With breaking, grids of two tiles
+// per SM and more at m = 2 to 4 (64^3, m = 3: 57.5 and 55.0; 72 x 80 x 90 with m = 1 26.6 and 27.5,
+// with m = 5 384 and 392). Below, ragged grids at m = 3 (37 x 29 x 41: 23.3 and 22.1, with breaking
+// 27.1 and 24.3) and, with breaking, at m = 2 (13.4 and 12.4; without 12.5 and 12.8): m = 1 has
+// few columns for the threads (9.3 and 10.6), and from m = 4 on half of the threads of a pair's
+// two would wait (m = 5: 45.6 and 46.6).
+static bool pmb_cols(const TileArgs &a, bool brk)
+{
+    const int m = a.g.m;
+    if (!cols_staging(a)) return false;
+    if (a.g.ntiles >= ROWS_MIN_TILES) return brk && m >= 2 && m <= 4;
+    return ragged(a) && (m == 3 || (m == 2 && brk));
+}
+
+template <int DIM, bool BRK, bool SPLIT, bool COLS>
+static int launch_fast_cols(const TileArgs &a, size_t smem, cudaStream_t st)
+{
+    PD_CUDA(smem_limit(pmb_fast<DIM, BRK, SPLIT, COLS>, smem));
+    pmb_fast<DIM, BRK, SPLIT, COLS><<<a.g.ntiles, a.g.T / 2 * a.split, smem, st>>>(a);
+    PD_CUDA(cudaGetLastError());
+    return PD_OK;
 }
 
 template <int DIM, bool BRK, bool SPLIT>
@@ -423,12 +444,12 @@ static int launch_fast_split(const TileArgs &a, cudaStream_t st)
     if (param_table(a.htab_a, a.ntab_a, a.g.ntiles, tp)) {
         PD_CUDA(smem_limit(pmb_fast_pt<DIM, BRK, SPLIT>, smem));
         pmb_fast_pt<DIM, BRK, SPLIT><<<a.g.ntiles, a.g.T / 2 * a.split, smem, st>>>(a, tp);
-    } else {
-        PD_CUDA(smem_limit(pmb_fast<DIM, BRK, SPLIT>, smem));
-        pmb_fast<DIM, BRK, SPLIT><<<a.g.ntiles, a.g.T / 2 * a.split, smem, st>>>(a);
+        PD_CUDA(cudaGetLastError());
+        return PD_OK;
     }
-    PD_CUDA(cudaGetLastError());
-    return PD_OK;
+    if constexpr (DIM == 3)
+        if (pmb_cols(a, BRK)) return launch_fast_cols<DIM, BRK, SPLIT, true>(a, smem, st);
+    return launch_fast_cols<DIM, BRK, SPLIT, false>(a, smem, st);
 }
 
 template <int DIM, bool BRK>
@@ -446,7 +467,7 @@ static int launch_fast(const TileArgs &a0, cudaStream_t st)
                   "breaking, or the CTA exceeds its limits", a.split, a.g.W);
         return PD_EINVAL;
     }
-    if (DIM == 3 && !BRK && a.rows && a.g.ntiles >= ROWS_MIN_TILES) return launch_rows_pmb(a, a.rows[1], st);
+    if (DIM == 3 && !BRK && a.rows && rows_pmb(a.g)) return launch_rows_pmb(a, a.rows[1], st);
     return a.split > 1 ? launch_fast_split<DIM, BRK, true>(a, st) : launch_fast_split<DIM, BRK, false>(a, st);
 }
 

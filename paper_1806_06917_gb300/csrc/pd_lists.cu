@@ -272,7 +272,7 @@ int build_tile_lists(const Geom &g, const Material &mat, const Tables &t, const 
     int rc = exclusive_scan(row_count, n, reinterpret_cast<long long *>(out->row_ptr), st);
     cudaError_t e = smem_limit(k_tile_rows, smem);
     if (rc == PD_OK && e == cudaSuccess) {
-        k_tile_rows<<<dim3(g.ntiles, std::min(8, std::max(1, 608 / g.ntiles))), 32 * LIST_WARPS, smem, st>>>(g, t.tile_org, tile_nbr, box_tab, box_cnt, nbox, t.stencil,
+        k_tile_rows<<<dim3(g.ntiles, std::min(8, std::max(1, 4 * SMS / g.ntiles))), 32 * LIST_WARPS, smem, st>>>(g, t.tile_org, tile_nbr, box_tab, box_cnt, nbox, t.stencil,
                                                              t.rank_of_slot, mask, stage_mask, out->row_ptr, out->col);
         e = cudaGetLastError();
     }

@@ -206,7 +206,7 @@ PD_PRAGMA_UNROLL(PD_DIL2_UNROLL)
 
 // Launch: one CTA per tile, T/2 threads (tiles of at least 2^7 points and two
 // stencil words).
-template <bool VOLCORR, bool PTAB>
+template <bool VOLCORR, bool PTAB, bool COLS>
 __device__ __forceinline__ void lps_dil_fast2_body(const TileArgs &a, int tile, const float4 *ptab)
 {
     const Geom &g = a.g;
@@ -223,7 +223,7 @@ __device__ __forceinline__ void lps_dil_fast2_body(const TileArgs &a, int tile, 
         for (int k = threadIdx.x; k < 3 * S; k += blockDim.x) tab[k] = __ldg(&a.tab_a[k]);
     load_nbr(a, tile, s_nbr);
     __syncthreads();
-    stage_pairs<!PTAB>(a, pb, org, tile, s_nbr, P4, P2, true);
+    stage_pairs<COLS>(a, pb, org, tile, s_nbr, P4, P2, true);
     __syncthreads();
     // 1/m~ of the tile's points, read by the epilogue (128^3 LPS pass 0.2167 -> 0.2151 ms)
     if (threadIdx.x == 0) l2_prefetch(a.minv32 + (size_t)tile * g.T, 4 * g.T);
@@ -445,10 +445,10 @@ __global__ void __launch_bounds__(256, PD_MINBLOCKS) lps_dil_fast(const TileArgs
     lps_dil_fast_body<VOLCORR, false>(a, blockIdx.x, nullptr);
 }
 
-template <bool VOLCORR>
+template <bool VOLCORR, bool COLS>
 __global__ void __launch_bounds__(256, PD_DIL2_MINBLOCKS) lps_dil_fast2(const TileArgs a)
 {
-    lps_dil_fast2_body<VOLCORR, false>(a, blockIdx.x, nullptr);
+    lps_dil_fast2_body<VOLCORR, false, COLS>(a, blockIdx.x, nullptr);
 }
 
 template <bool VOLCORR>
@@ -469,7 +469,7 @@ template <bool VOLCORR>
 __global__ void __launch_bounds__(256, PD_DIL2_MINBLOCKS)
     lps_dil_fast2_pt(const __grid_constant__ TileArgs a, const __grid_constant__ ParamTab tp)
 {
-    lps_dil_fast2_body<VOLCORR, true>(a, blockIdx.x, tp.e);
+    lps_dil_fast2_body<VOLCORR, true, false>(a, blockIdx.x, tp.e);
 }
 
 template <bool VOLCORR>

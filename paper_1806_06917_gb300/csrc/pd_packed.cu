@@ -108,8 +108,8 @@ static __device__ __forceinline__ void pk_lps_force(const TileArgs &a, int tile,
 }
 static __device__ __forceinline__ void pk_pmb3s(const TileArgs &a, int tile) { pmb_fast_body<3, false, true, false, false>(a, tile, nullptr); }
 static __device__ __forceinline__ void pk_pmb3(const TileArgs &a, int tile) { pmb_fast_body<3, false, false, false, false>(a, tile, nullptr); }
-static __device__ __forceinline__ void pk_pmb2s(const TileArgs &a, int tile) { pmb_fast_body<2, false, true, false>(a, tile, nullptr); }
-static __device__ __forceinline__ void pk_pmb2(const TileArgs &a, int tile) { pmb_fast_body<2, false, false, false>(a, tile, nullptr); }
+static __device__ __forceinline__ void pk_pmb2s(const TileArgs &a, int tile) { pmb_fast_body<2, false, true, false, false>(a, tile, nullptr); }
+static __device__ __forceinline__ void pk_pmb2(const TileArgs &a, int tile) { pmb_fast_body<2, false, false, false, false>(a, tile, nullptr); }
 
 __global__ void __launch_bounds__(PACK_THREADS, 2) pd_packed_round(const __grid_constant__ PackTable t, int round)
 {

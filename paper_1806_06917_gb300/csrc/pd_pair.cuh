@@ -267,6 +267,10 @@ __device__ __forceinline__ void for_pair_slots(const TileArgs &a, const PairBox 
     }
 }
 
+// Where staging by columns is possible, and whether the grid has tiles without the box map.
+inline bool cols_staging(const TileArgs &a) { return a.nbr_ok && a.g.dim == 3 && a.g.L == 9; }
+inline bool ragged(const TileArgs &a) { return !a.box_map || a.g.nx % 8 || a.g.ny % 8 || a.g.nz % 8; }
+
 // Stage the box column by column: a thread takes a column (x, y) and loads each of
 // its points that some bond of the tile reaches once (|z| limited by the column's
 // distance from the tile; the pair-wise staging loads the points of shared planes
@@ -356,15 +360,17 @@ __device__ __forceinline__ void stage_columns(const TileArgs &a, const int4 &org
 // changes nothing in the one-wave 64^3 PMB step, whose staging waits on memory
 // more than it issues. The coordinate loop is kept apart from for_pair_slots:
 // through it the 2D NP kernel (443^2, m = 20, no map) measured 1 % slower.
+// COLS: by columns, on grids of two tiles an SM and more and in edge tiles, whose other form
+// computes every entry's coordinates. A template choice, since the code beside the other
+// form's costs spills on grids that have neither (40^3 PMB step 0.0199 -> 0.0203 ms). (nbr_ok
+// and bz hold wherever COLS is chosen; without them here the compiler's code took 1 to 3 %
+// longer with breaking.)
 template <bool COLS = false>
 __device__ __forceinline__ void stage_pairs(const TileArgs &a, const PairBox &pb, const int4 &org, int tile,
                                             const int *s_nbr, float4 *P4, float2 *P2, bool use_map)
 {
     const Ref32 ref = tile_ref32(a, tile);
     const float inv_h = (float)a.inv_h;
-    // Columns on grids of two tiles an SM and more (64^3 PMB with breaking 0.0577 -> 0.0553
-    // ms) and in edge tiles, whose other form computes every entry's coordinates (37 x 29 x
-    // 41: 0.0484 -> 0.0469 ms); a single whole tile an SM measured 1-2 % slower with them.
     if (COLS && a.nbr_ok && a.g.bz == 8 && (a.g.ntiles >= ROWS_MIN_TILES || !box_mapped(a, org))) {
         stage_columns<false, 1>(a, org, ref, s_nbr, nullptr, P4, P2, nullptr);
         return;

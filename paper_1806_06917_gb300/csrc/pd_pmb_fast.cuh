@@ -244,11 +244,11 @@ __device__ __forceinline__ void pair_split_sum(const TileArgs &a, float2 *red, i
 // blockIdx.x; the request server's packed kernel (pd_packed.cu) runs it for the
 // tiles of its work items, with a in shared memory.
 // PTAB: the table is read from ptab (a kernel parameter) instead of shared memory.
-// COLS: grids of many or ragged tiles are staged by columns (stage_pairs). The packed
-// kernel leaves that out: beside its other bodies in 64 registers it spilled 496 bytes a
-// thread instead of 196, which every request paid for (128^3 LPS alone 0.573 -> 0.617 ms a
-// step, twelve mixed requests 15.5 -> 16.2 ms).
-template <int DIM, bool BRK, bool SPLIT, bool PTAB, bool COLS = DIM == 3 && !PTAB>
+// COLS: staged by columns (stage_pairs; pmb_cols below). The packed kernel leaves that out:
+// beside its other bodies in 64 registers it spilled 496 bytes a thread instead of 196, which
+// every request paid for (128^3 LPS alone 0.573 -> 0.617 ms a step, twelve mixed requests 15.5
+// -> 16.2 ms).
+template <int DIM, bool BRK, bool SPLIT, bool PTAB, bool COLS>
 __device__ __forceinline__ void pmb_fast_body(const TileArgs &a, int tile, const float4 *ptab)
 {
     const Geom &g = a.g;
@@ -357,18 +357,18 @@ __device__ __forceinline__ void pmb_fast_body(const TileArgs &a, int tile, const
     }
 }
 
-template <int DIM, bool BRK, bool SPLIT>
+template <int DIM, bool BRK, bool SPLIT, bool COLS>
 __global__ void __launch_bounds__(SPLIT ? 1024 : 256, SPLIT ? 1 : PD_MINBLOCKS)
     pmb_fast(const __grid_constant__ TileArgs a)
 {
-    pmb_fast_body<DIM, BRK, SPLIT, false>(a, blockIdx.x, nullptr);
+    pmb_fast_body<DIM, BRK, SPLIT, false, COLS>(a, blockIdx.x, nullptr);
 }
 
 template <int DIM, bool BRK, bool SPLIT>
 __global__ void __launch_bounds__(SPLIT ? 1024 : 256, SPLIT ? 1 : PD_MINBLOCKS)
     pmb_fast_pt(const __grid_constant__ TileArgs a, const __grid_constant__ ParamTab tp)
 {
-    pmb_fast_body<DIM, BRK, SPLIT, true>(a, blockIdx.x, tp.e);
+    pmb_fast_body<DIM, BRK, SPLIT, true, false>(a, blockIdx.x, tp.e);
 }
 
 }  // namespace pdk

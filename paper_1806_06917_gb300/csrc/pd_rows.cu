@@ -38,7 +38,7 @@ static int go_parts(const TileArgs &a, const RowArgs &ra, cudaStream_t st)
 {
     // the table as a kernel parameter on grids of several waves, as for the word-wise
     // kernels (pd_force_pmb.cu)
-    const bool pt = ra.ntab <= ROWS_PTAB && a.g.ntiles >= 2048;
+    const bool pt = ra.ntab <= ROWS_PTAB && a.g.ntiles >= PTAB_MIN_TILES;
     const size_t smem = rows_smem(ra, LAW == ROW_FRC, pt);
     if (pt) {
         static thread_local RowTab tab;

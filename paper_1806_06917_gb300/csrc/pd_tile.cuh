@@ -401,12 +401,35 @@ __device__ __forceinline__ void split_bits(double u, float &hi, float &lo)
 // entry, then one per segment and one of zeros.
 constexpr int ROWS_PTAB = 280;      // float4 that fit the kernel parameter: m <= 3 (122 entries, 32 segments)
 constexpr int ROWS_PLANES = 20;     // pair planes of the box: 4 + 2m, m <= 8
-// Where the row-wise passes take over: from two tiles per SM on (40^3 PMB, 125 tiles:
-// 0.0201 ms word-wise and 0.0247 row-wise; 64^3, 512 tiles: 0.0493 and 0.0468), the LPS
-// force pass, at 128 registers and two CTAs per SM, from more than one tile per SM on
-// (45 x 37 x 52, 210 tiles: 0.0369 and 0.0342; 33 x 45 x 27 with m = 4, 120 tiles: 0.0389
-// and 0.0427). Below, the word-wise kernels' twice as many threads per tile count.
-constexpr int ROWS_MIN_TILES = 304, ROWS_MIN_TILES_FRC = 153;
+// The rules of the dispatch count tiles per SM of a GB300.
+constexpr int SMS = 152;
+// Grids of several waves of tiles: there the stencil tables go into the kernel parameter.
+constexpr int PTAB_MIN_TILES = 2048;
+// Where the row-wise passes take over (us a step, word-wise and row-wise):
+// - PMB and the dilatation from two tiles per SM on (40^3 PMB, 125 tiles: 20.1 and 24.7; 64^3,
+//   512 tiles: 49.3 and 46.8). Below, the word-wise kernels have twice as many threads per
+//   tile.
+// - PMB at m = 3 (two ranges: 128^3 322 and 255). Shorter horizons leave segments of one and
+//   two bonds (m = 1: 128^3 96 and 110; m = 2: 80^3 32.3 and 33.9, 128^3 132 and 139), and at
+//   longer ones the word-wise kernel runs two threads a pair (m = 4: 64^3 88.7 and 99.6;
+//   m = 5: 169 and 176).
+// - but not from 4.5 to 5 tiles per SM: the four CTAs of an SM end together here, so that the
+//   last tiles gather on a few SMs (693 tiles 60.4 and 60.0, 704 to 756 60.3 and 65.8, 768 69.6
+//   and 66.4).
+// - LPS from m = 2 on (m = 1: 56^3 0.94 of the speed, 128^3 0.98).
+// - the LPS force pass, at 128 registers and two CTAs per SM, from more than one tile per SM
+//   on (45 x 37 x 52, 210 tiles: 36.9 and 34.2; 33 x 45 x 27 with m = 4, 120 tiles: 38.9 and 42.7),
+//   where two CTAs' boxes fit in an SM (m = 5, one CTA: 48^3 210 and 227).
+constexpr int ROWS_MIN_TILES = 2 * SMS, ROWS_MIN_TILES_FRC = SMS + 1;
+inline bool rows_pmb(const Geom &g)
+{
+    return g.m == 3 && g.ntiles >= ROWS_MIN_TILES && !(2 * g.ntiles > 9 * SMS && g.ntiles <= 5 * SMS);
+}
+inline bool rows_dil(const Geom &g) { return g.m >= 2 && g.ntiles >= ROWS_MIN_TILES; }
+inline bool rows_frc(const Geom &g, size_t smem)
+{
+    return g.ntiles >= ROWS_MIN_TILES_FRC && 2 * (smem + 1024) <= 228 * 1024;
+}
 struct RowArgs {
     const float4 *tab, *htab;       // device table and its host copy
     int ntab, nseg;                 // float4 of the table, segments
