@@ -397,6 +397,19 @@ typedef struct {
  * kept until pd_destroy. Synchronous. */
 int pd_solve_static(pd_sim *sim, const pd_newton_opts *opts, pd_newton_stats *stats, void *stream);
 
+/* How pd_solve_static runs GMRES with the cached tangent and no preconditioner (the other
+ * solves have one form). GRID: a cycle in one cooperative launch, whose blocks wait for
+ * each other at most wait_limit_ms at a time (0 = 2000); GRAPH: a kernel per operation,
+ * in captured graphs; AUTO (the default): GRID, and GRAPH from the cycle on for which the
+ * launch is not possible or a wait runs out. GRID alone fails then with PD_ENOTREADY or
+ * PD_ETIMEOUT (u is the last Newton iterate). Both forms solve the same Krylov spaces; their
+ * sums differ by rounding. test_stall: tests only, else 0: a block of the launch stays away,
+ * so that the others' wait runs out. Holds for the simulation until set again. */
+#define PD_GMRES_AUTO 0
+#define PD_GMRES_GRAPH 1
+#define PD_GMRES_GRID 2
+int pd_set_gmres_form(pd_sim *sim, int form, int wait_limit_ms, int test_stall);
+
 /* ------------------------------------------------------------------- serving */
 
 /* A request server: independent simulations submitted at any time, run

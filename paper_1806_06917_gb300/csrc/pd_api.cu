@@ -189,6 +189,7 @@ struct pd_sim {
     size_t nk_basis_n = 0, nk_partial_n = 0, nk_dsc_n = 0;
     void *nk_tan = nullptr;         // per-bond tangent cache
     size_t nk_tan_n = 0;
+    int gm_form = PD_GMRES_AUTO, gm_wait_ms = 0, gm_stall = 0;      // pd_set_gmres_form
     // graphs: [start parity]
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
 };
@@ -1882,6 +1883,19 @@ int pd_vjp(pd_sim *s, const double *u_lin, const double *v, double *out, unsigne
     return tangent(s, u_lin, v, out, flags, 1, stream);
 }
 
+int pd_set_gmres_form(pd_sim *s, int form, int wait_limit_ms, int test_stall)
+{
+    CHECK_SIM(s);
+    if (form < PD_GMRES_AUTO || form > PD_GMRES_GRID || wait_limit_ms < 0 || (test_stall != 0 && test_stall != 1)) {
+        set_error("pd_set_gmres_form: unknown form, negative limit or test_stall other than 0 and 1");
+        return PD_EINVAL;
+    }
+    s->gm_form = form;
+    s->gm_wait_ms = wait_limit_ms;
+    s->gm_stall = test_stall;
+    return PD_OK;
+}
+
 int pd_solve_static(pd_sim *s, const pd_newton_opts *opts, pd_newton_stats *stats, void *stream)
 {
     CHECK_BUILT(s);
@@ -1934,7 +1948,8 @@ int pd_solve_static(pd_sim *s, const pd_newton_opts *opts, pd_newton_stats *stat
         s->nk_tan_n = tan_bytes;
     }
     if ((rc = ensure_cap(s)) != PD_OK) return rc;
-    KrylovWork wk{s->nk_basis, s->nk_tmp, s->nk_aux, s->nk_partial, s->nk_dsc, s->cap_stream};
+    KrylovWork wk{s->nk_basis, s->nk_tmp, s->nk_aux, s->nk_partial, s->nk_dsc, s->cap_stream,
+                  s->gm_form, (s->gm_wait_ms ? s->gm_wait_ms : 2000) * 1000000LL, s->gm_stall};
     const TanOp tan = cached ? tangent_op(g, s->precision, s->nk_tan, s->user_of_slot, s->bc_kind) : TanOp{};
     KrylovOp op{cached ? nk_apply_cached : nk_apply, s, jacobi ? nk_precond : nullptr, cached ? &tan : nullptr};
     const unsigned nbs = (unsigned)((g.nslots + 255) / 256);

@@ -174,7 +174,10 @@ struct KrylovWork {
     double *aux;        // 2 * n (preconditioned solves)
     double *partial;    // krylov_partial_doubles(n, restart)
     double *dsc;        // krylov_dsc_doubles(...)
-    cudaStream_t cap;   // a stream for graph capture (CG), or null
+    cudaStream_t cap;   // a stream for graph capture, or null
+    int form;           // PD_GMRES_*
+    long long wait_ns;  // limit of one wait of the grid form
+    int stall;          // tests: a wait of the grid form runs out
 };
 struct KrylovStats {
     int iters;

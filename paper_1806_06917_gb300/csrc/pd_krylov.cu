@@ -11,7 +11,9 @@
 // residual estimate from the Arnoldi vector's norm; CG's alpha and beta are
 // formed from p.Ap and r.r. The host reads the scalars back once per chunk of
 // iterations (GM_CHUNK Arnoldi steps, CG_CHUNK CG iterations), each chunk
-// replayed as a captured CUDA graph.
+// replayed as a captured CUDA graph; with the cached tangent and no
+// preconditioner a GMRES cycle is one launch instead (pd_krylov_grid.cu), read
+// back once.
 #include <vector>
 
 #include "pd_krylov.cuh"
@@ -185,6 +187,18 @@ __global__ void k_scale_dev(const double *d, int idx, double *y, long long n)
 // rotations: solve A x = b from x = 0 until ||b - A x|| <= rtol ||b||. With a
 // preconditioner M it is right-preconditioned (Arnoldi on A M^-1, x += M^-1 V y),
 // so the residual it monitors is the one of A x = b.
+// Whether the one-launch form is the faster one: not where an FP32 tangent's product moves
+// more than 20 times what the Gram-Schmidt passes of an average step do. One block of 1024
+// threads an SM reads the tangent less fast than the product's own kernel (restart 3, us a
+// step, launch and kernels: 40^3 with m = 3 269 and 254, 64^3 829 and 809, 400^2 with m = 8 561 and
+// 548; restart 10: 221, 704, 469 and 221, 711, 472).
+static bool grid_pays(const TanOp &t, int restart)
+{
+    const long long product = (long long)t.S * (4 * (t.dim == 3 ? 6 : 3) + 4);      // bytes a slot
+    const long long passes = 4LL * restart / 2 * t.dim * (long long)sizeof(double);
+    return t.fp64 || product <= 20 * passes;
+}
+
 int krylov_gmres(const KrylovOp &op, const double *b, double *x, long long n, int restart, int maxit, double rtol,
                  KrylovWork &wk, KrylovStats *stats, cudaStream_t st)
 {
@@ -274,6 +288,7 @@ int krylov_gmres(const KrylovOp &op, const double *b, double *x, long long n, in
     std::vector<double> init(L.size(), 0.0);
     double back[8];
     bool first = true;
+    bool grid_form = op.tan && !pc && (wk.form == PD_GMRES_GRID || (wk.form == PD_GMRES_AUTO && grid_pays(*op.tan, m)));
     while (true) {
         // r = b - A x  (x = 0 on the first cycle)
         double beta;
@@ -301,24 +316,29 @@ int krylov_gmres(const KrylovOp &op, const double *b, double *x, long long n, in
         const int steps = std::min(m, maxit - stats->iters);
         int k = 0;
         bool done = false;
-        bool grid = false;
-        if (op.tan && !pc) {
-            rc = gmres_grid(*op.tan, V, n, c.partial, c.dsc, m, steps, st);
-            grid = rc == PD_OK;
+        if (grid_form) {
+            rc = gmres_grid(*op.tan, V, n, c.partial, c.dsc, m, steps, wk.wait_ns, wk.stall, st);
             if (rc != PD_OK && rc != PD_ENOTREADY) return rc;
-            if (grid) {
-                unsigned sy = 0;
+            unsigned sy = 0;
+            if (rc == PD_OK) {
                 PD_CUDA(cudaMemcpyAsync(back, c.dsc + L.sc, sizeof(back), cudaMemcpyDeviceToHost, st));
                 PD_CUDA(cudaMemcpyAsync(&sy, c.dsc + L.size(), sizeof(sy), cudaMemcpyDeviceToHost, st));
                 PD_CUDA(cudaStreamSynchronize(st));
-                if (sy >> 31) {   // a wait that ran out
-                    set_error("GMRES: a wait of the grid kernel ran out");
-                    return PD_ETIMEOUT;
-                }
                 k = (int)back[GM_K];
+                if (sy >> 31) rc = PD_ETIMEOUT;
+            }
+            if (rc != PD_OK && wk.form == PD_GMRES_GRID) {
+                set_error(rc == PD_ETIMEOUT ? "GMRES: a wait of the grid kernel ran out" :
+                                              "GMRES: the cooperative launch is not possible");
+                return rc;
+            }
+            if (rc != PD_OK) {      // this cycle again (V_0 is untouched) and the rest, kernel by kernel
+                grid_form = false;
+                k = 0;
+                PD_CUDA(cudaMemcpyAsync(c.dsc, init.data(), sizeof(double) * init.size(), cudaMemcpyHostToDevice, st));
             }
         }
-        for (int j0 = 0; j0 < steps && !done && !grid; j0 += GM_CHUNK) {
+        for (int j0 = 0; j0 < steps && !done && !grid_form; j0 += GM_CHUNK) {
             const int j1 = std::min(steps, j0 + GM_CHUNK);
             cudaGraphExec_t ge = j1 == std::min(m, j0 + GM_CHUNK) ? chunk_graph(j0) : nullptr;
             if (ge) {

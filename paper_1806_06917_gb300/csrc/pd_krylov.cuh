@@ -34,9 +34,10 @@ __device__ __forceinline__ double block_sum(double v, double *red)
 // Device layout of GMRES's small arrays in dsc (m = restart): the dot results
 // [0, m+1), the Hessenberg matrix H (column-major, (m+1) x m), the rotations cs
 // and sn, the rotated right-hand side g (m+1), the solution y of the small
-// triangular system (m), and the scalars. The host enqueues GM_CHUNK Arnoldi
-// steps at a time and reads back once per chunk; a step after the one that
-// met the target (or broke down) changes nothing that the update of x uses.
+// triangular system (m), and the scalars. The host reads the scalars back once
+// per chunk of Arnoldi steps (a kernel per operation) or once per cycle (one
+// launch); a step after the one that met the target (or broke down) changes
+// nothing that the update of x uses.
 struct GmLayout {
     int m, H, cs, sn, g, y, sc;
     __host__ __device__ explicit GmLayout(int m_)
@@ -97,6 +98,7 @@ constexpr int GRID_MAX = 256;
 // The grid form: steps 0 .. steps - 1 of a GMRES cycle from V_0 and the scalars in d, whose
 // last double (after GmLayout's) is the barrier. PD_ENOTREADY where the launch is not possible
 // (nothing has run).
-int gmres_grid(const TanOp &t, double *V, long long n, double *partial, double *d, int m, int steps, cudaStream_t st);
+int gmres_grid(const TanOp &t, double *V, long long n, double *partial, double *d, int m, int steps, long long wait_ns,
+               int stall, cudaStream_t st);
 
 }  // namespace pdk

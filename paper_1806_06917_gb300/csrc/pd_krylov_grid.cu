@@ -27,14 +27,12 @@ constexpr int GSEG = 8;                   // warps per product at most
 
 // ------------------------------------------------------------ grid barrier
 
-constexpr long long GRID_WAIT_NS = 2000000000LL;
-
 // Every block of the cooperative launch arrives; bounded: a block that has waited
-// GRID_WAIT_NS sets the word's top bit and returns false, and so does every block that finds
-// it set (the count stays below it: 152 blocks, 7 arrivals a step, a few thousand steps).
+// wait_ns sets the word's top bit and returns false, and so does every block that finds
+// it set (the count stays below it: 256 blocks at most, 7 arrivals a step, 500 steps).
 constexpr unsigned GRID_FAILED = 0x80000000u;
 
-__device__ __forceinline__ bool grid_barrier(unsigned *sync, unsigned &target)
+__device__ __forceinline__ bool grid_barrier(unsigned *sync, unsigned &target, long long wait_ns)
 {
     __shared__ int s_ok;
     target += gridDim.x;
@@ -49,7 +47,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned *sync, unsigned &target)
             if (polls % 64) continue;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
             if (polls == 0) t0 = t;
-            if (t - t0 > GRID_WAIT_NS) {
+            if (t - t0 > wait_ns) {
                 v = atomicOr(sync, GRID_FAILED) | GRID_FAILED;
                 break;
             }
@@ -156,11 +154,15 @@ __device__ __forceinline__ double slices_total(const double *p, int nb)
     return acc;
 }
 
-// Arnoldi steps 0 .. steps - 1 of a cycle (V_0 and the scalars are set).
+// Arnoldi steps 0 .. steps - 1 of a cycle (V_0 and the scalars are set). V_0 stays as it is,
+// so that a cycle whose wait ran out can be run again. stall (tests): block 0 does not take
+// part, so that the others' first wait runs out.
 template <class R, int DIM>
 __global__ void __launch_bounds__(GT, 1) k_gmres_grid(const __grid_constant__ TanOp t, double *V, long long n,
-                                                     double *partial, double *d, int m, int steps, unsigned *sync)
+                                                     double *partial, double *d, int m, int steps, unsigned *sync,
+                                                     long long wait_ns, int stall)
 {
+    if (stall && blockIdx.x == 0) return;
     extern __shared__ double sm[];          // h (m + 1), the products' sums; the last block: 3 (m + 1)
     double *h = sm, *buf = sm + m + 1;
     __shared__ double s_norm2, s_inv;
@@ -175,11 +177,11 @@ __global__ void __launch_bounds__(GT, 1) k_gmres_grid(const __grid_constant__ Ta
         double *w = V + (long long)(j + 1) * n;
         if (!last) apply_groups<R, DIM>(t, V + (long long)j * n, w, me, own);
         else if (j > 0) gm_givens(d, m, j - 1, s_norm2, buf);
-        if (!grid_barrier(sync, target)) return;
+        if (!grid_barrier(sync, target, wait_ns)) return;
         if (j > 0 && __ldcg(&d[L.sc + GM_DONE]) != 0.0) return;
         for (int pass = 0; pass < 2; ++pass) {
             if (!last) slice_dots(V, j + 1, w, n, lo, hi, nseg, buf, partial + me, own);
-            if (!grid_barrier(sync, target)) return;
+            if (!grid_barrier(sync, target, wait_ns)) return;
             if (warp == 0)
                 for (int i = me; i <= j; i += own + 1) {
                     const double x = slices_total(partial + (long long)i * own, own);
@@ -189,7 +191,7 @@ __global__ void __launch_bounds__(GT, 1) k_gmres_grid(const __grid_constant__ Ta
                         *H = pass ? *H + x : x;
                     }
                 }
-            if (!grid_barrier(sync, target)) return;
+            if (!grid_barrier(sync, target, wait_ns)) return;
             for (int i = threadIdx.x; i <= j; i += GT) h[i] = __ldcg(&d[i]);
             __syncthreads();
             for (long long e = lo + threadIdx.x; e < hi; e += GT) {
@@ -200,7 +202,7 @@ __global__ void __launch_bounds__(GT, 1) k_gmres_grid(const __grid_constant__ Ta
             }
         }
         if (!last) slice_dots(w, 1, w, n, lo, hi, nnorm, buf, partial + me, own);
-        if (!grid_barrier(sync, target)) return;
+        if (!grid_barrier(sync, target, wait_ns)) return;
         if (warp == 0) {
             const double x = slices_total(partial, own);
             if (threadIdx.x == 0) {    // one thread: a square root and a quotient by every warp took 5 us
@@ -212,7 +214,7 @@ __global__ void __launch_bounds__(GT, 1) k_gmres_grid(const __grid_constant__ Ta
         __syncthreads();
         const double inv = s_inv;
         for (long long e = lo + threadIdx.x; e < hi; e += GT) w[e] = inv * __ldcg(&w[e]);
-        if (!grid_barrier(sync, target)) return;
+        if (!grid_barrier(sync, target, wait_ns)) return;
     }
     if (last) gm_givens(d, m, steps - 1, s_norm2, buf);
 }
@@ -239,10 +241,11 @@ static int go(F *k, int smem, void **args, unsigned *sync, cudaStream_t st)
                                                                                  : cuda_fail(e, "cooperative launch");
 }
 
-int gmres_grid(const TanOp &t, double *V, long long n, double *partial, double *d, int m, int steps, cudaStream_t st)
+int gmres_grid(const TanOp &t, double *V, long long n, double *partial, double *d, int m, int steps, long long wait_ns,
+               int stall, cudaStream_t st)
 {
     unsigned *sync = reinterpret_cast<unsigned *>(d + GmLayout(m).size());
-    void *args[] = {(void *)&t, &V, &n, &partial, &d, &m, &steps, &sync};
+    void *args[] = {(void *)&t, &V, &n, &partial, &d, &m, &steps, &sync, &wait_ns, &stall};
     const int smem = (m + 1 + std::max(GSEG * (m + 1), GW)) * (int)sizeof(double);
     if (t.fp64) return go(t.dim == 3 ? k_gmres_grid<double, 3> : k_gmres_grid<double, 2>, smem, args, sync, st);
     return go(t.dim == 3 ? k_gmres_grid<float, 3> : k_gmres_grid<float, 2>, smem, args, sync, st);

@@ -27,6 +27,7 @@ PD_JVP_MASK_DIRICHLET = 1
 PD_KRYLOV_GMRES, PD_KRYLOV_CG = 0, 1
 PD_TANGENT_CACHED, PD_TANGENT_JVP = 0, 1
 PD_PRECOND_NONE, PD_PRECOND_BLOCK_JACOBI = 0, 1
+PD_GMRES_AUTO, PD_GMRES_GRAPH, PD_GMRES_GRID = 0, 1, 2
 PD_INTEGRATOR_VERLET, PD_INTEGRATOR_CD = 0, 1
 PD_STATE_F64, PD_STATE_DF = 0, 1          # pd_run.state of a PD_FP32C simulation
 PD_SERVE_PACKED, PD_SERVE_STREAMS = 0, 1   # pd_server_opts.mode
@@ -126,6 +127,7 @@ _SIGS = {
     "pd_vjp": [_P, _P, _P, _P, ctypes.c_uint, _P],
     "pd_energy": [_P, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double), _P],
     "pd_solve_static": [_P, ctypes.POINTER(pd_newton_opts), ctypes.POINTER(pd_newton_stats), _P],
+    "pd_set_gmres_form": [_P, ctypes.c_int, ctypes.c_int, ctypes.c_int],
     "pd_server_create": [ctypes.POINTER(_P), ctypes.POINTER(pd_server_opts)],
     "pd_server_destroy": [_P],
     "pd_submit": [_P, ctypes.POINTER(pd_request), ctypes.POINTER(ctypes.c_uint64)],
@@ -396,6 +398,11 @@ def pd_solve_static(sim: Sim, opts: pd_newton_opts | None = None, stream=None) -
     _check(_lib.pd_solve_static(sim.h, ctypes.byref(opts) if opts is not None else None, ctypes.byref(st),
                                 _stream(stream)))
     return {k: getattr(st, k) for k, _ in pd_newton_stats._fields_}
+
+
+def pd_set_gmres_form(sim: Sim, form: int = PD_GMRES_AUTO, wait_limit_ms: int = 0, test_stall: int = 0) -> None:
+    """How pd_solve_static runs GMRES with the cached tangent and no preconditioner (PD_GMRES_*)."""
+    _check(_lib.pd_set_gmres_form(sim.h, int(form), int(wait_limit_ms), int(test_stall)))
 
 
 def _result(r: pd_result) -> dict:
