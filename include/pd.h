@@ -333,8 +333,9 @@ int pd_tune(const pd_grid *grid, const pd_material *mat, const pd_run *run, int3
 int pd_jvp(pd_sim *sim, const double *u_lin, const double *w, double *out,
            unsigned flags, void *stream);
 
-/* Adjoint (vector-Jacobian) product out = K^T v, computed by its own kernel in
- * the transposed gather form (K^T v)_i = sum_j D_ij (V_i v_j - V_j v_i) V_ij.
+/* Adjoint (vector-Jacobian) product out = K^T v, the transposed gather
+ * (K^T v)_i = sum_j D_ij (V_i v_j - V_j v_i) V_ij. FP32C evaluates D from the other end
+ * of the bond; in FP64 the gather has the same terms as pd_jvp's and is the same kernel.
  * Same arguments and errors as pd_jvp. */
 int pd_vjp(pd_sim *sim, const double *u_lin, const double *v, double *out,
            unsigned flags, void *stream);

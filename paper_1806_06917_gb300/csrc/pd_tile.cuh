@@ -1,6 +1,6 @@
 // pd_tile.cuh -- machinery shared by the tile kernels (force, step, tangent,
-// energy): packed arithmetic on P points per thread, the horizon stencil as
-// compile-time constants, and shared-memory staging of a tile's halo box.
+// energy): FP64 roots and quotients, shared-memory staging of a tile's halo box,
+// the rules of the dispatch and the kernels' arguments.
 //
 // A CTA owns one tile (a Morton brick of T = 2^L lattice points). It stages the
 // displacements of the brick plus an m-wide halo into shared memory as a dense
@@ -18,8 +18,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <utility>
-
 #include "pd_internal.cuh"
 
 // float4 words per stencil entry of the FP32C NP / LP table (np_word in
@@ -27,88 +25,6 @@
 #define NP_TAB_WORDS(dim) ((dim) == 3 ? 3 : 2)
 
 namespace pdk {
-
-// ----------------------------------------------------------- packed values
-
-// P values of type R, one per point handled by the thread. For float with P = 2
-// every elementwise op is one Blackwell packed-FP32 instruction (f32x2).
-template <class R, int P>
-struct Pk {
-    R v[P];
-};
-
-template <class R, int P>
-__device__ __forceinline__ Pk<R, P> splat(R x)
-{
-    Pk<R, P> r;
-#pragma unroll
-    for (int p = 0; p < P; ++p) r.v[p] = x;
-    return r;
-}
-
-#define PD_PK_BINOP(NAME, EXPR)                                                   \
-    template <class R, int P>                                                     \
-    __device__ __forceinline__ Pk<R, P> NAME(const Pk<R, P> &a, const Pk<R, P> &b) \
-    {                                                                             \
-        Pk<R, P> r;                                                               \
-        _Pragma("unroll") for (int p = 0; p < P; ++p) r.v[p] = EXPR;              \
-        return r;                                                                 \
-    }
-PD_PK_BINOP(padd, a.v[p] + b.v[p])
-PD_PK_BINOP(psub, a.v[p] - b.v[p])
-PD_PK_BINOP(pmul, a.v[p] * b.v[p])
-#undef PD_PK_BINOP
-
-template <class R, int P>
-__device__ __forceinline__ Pk<R, P> pfma(const Pk<R, P> &a, const Pk<R, P> &b, const Pk<R, P> &c)
-{
-    Pk<R, P> r;
-#pragma unroll
-    for (int p = 0; p < P; ++p) r.v[p] = fma(a.v[p], b.v[p], c.v[p]);
-    return r;
-}
-
-// float x 2: packed instructions.
-__device__ __forceinline__ float2 f2(const Pk<float, 2> &a) { return make_float2(a.v[0], a.v[1]); }
-__device__ __forceinline__ Pk<float, 2> pk2(float2 a)
-{
-    Pk<float, 2> r;
-    r.v[0] = a.x;
-    r.v[1] = a.y;
-    return r;
-}
-template <>
-__device__ __forceinline__ Pk<float, 2> padd(const Pk<float, 2> &a, const Pk<float, 2> &b)
-{
-    return pk2(__fadd2_rn(f2(a), f2(b)));
-}
-template <>
-__device__ __forceinline__ Pk<float, 2> psub(const Pk<float, 2> &a, const Pk<float, 2> &b)
-{
-    return pk2(__fadd2_rn(f2(a), make_float2(-b.v[0], -b.v[1])));
-}
-template <>
-__device__ __forceinline__ Pk<float, 2> pmul(const Pk<float, 2> &a, const Pk<float, 2> &b)
-{
-    return pk2(__fmul2_rn(f2(a), f2(b)));
-}
-template <>
-__device__ __forceinline__ Pk<float, 2> pfma(const Pk<float, 2> &a, const Pk<float, 2> &b,
-                                             const Pk<float, 2> &c)
-{
-    return pk2(__ffma2_rn(f2(a), f2(b), f2(c)));
-}
-
-// x + k and x * k for a compile-time or uniform scalar k.
-template <class R, int P>
-__device__ __forceinline__ Pk<R, P> padds(const Pk<R, P> &a, R k) { return padd(a, splat<R, P>(k)); }
-template <class R, int P>
-__device__ __forceinline__ Pk<R, P> pmuls(const Pk<R, P> &a, R k) { return pmul(a, splat<R, P>(k)); }
-template <class R, int P>
-__device__ __forceinline__ Pk<R, P> pfmas(const Pk<R, P> &a, R k, const Pk<R, P> &c)
-{
-    return pfma(a, splat<R, P>(k), c);
-}
 
 // ------------------------------------------------------------ FP64 helpers
 
@@ -169,41 +85,10 @@ __device__ __forceinline__ double prsqrt1(double q) { return f64_rsqrt(q); }
 __device__ __forceinline__ float pdiv1(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double pdiv1(double a, double b) { return f64_div(a, b); }
 
-template <class R, int P>
-__device__ __forceinline__ Pk<R, P> prsqrt(const Pk<R, P> &q)
-{
-    Pk<R, P> r;
-#pragma unroll
-    for (int p = 0; p < P; ++p) r.v[p] = prsqrt1(q.v[p]);
-    return r;
-}
-template <class R, int P>
-__device__ __forceinline__ Pk<R, P> pdiv(const Pk<R, P> &a, const Pk<R, P> &b)
-{
-    Pk<R, P> r;
-#pragma unroll
-    for (int p = 0; p < P; ++p) r.v[p] = pdiv1(a.v[p], b.v[p]);
-    return r;
-}
-
 // ------------------------------------------------------------------ stencil
 
-// k-th offset of the horizon stencil {d : 0 < |d|^2 <= m^2}, ordered by
-// (dz, dy, dx) ascending; comp 0..2 = dx, dy, dz, comp 3 = |d|^2.
-__host__ __device__ constexpr int stencil_entry(int dim, int m, int k, int comp)
-{
-    int idx = 0;
-    for (int dz = (dim == 3 ? -m : 0); dz <= (dim == 3 ? m : 0); ++dz)
-        for (int dy = -m; dy <= m; ++dy)
-            for (int dx = -m; dx <= m; ++dx) {
-                int d2 = dx * dx + dy * dy + dz * dz;
-                if (d2 == 0 || d2 > m * m) continue;
-                if (idx == k) return comp == 0 ? dx : comp == 1 ? dy : comp == 2 ? dz : d2;
-                ++idx;
-            }
-    return 0;
-}
-
+// Offsets of the horizon stencil {d : 0 < |d|^2 <= m^2}, which is ordered by (dz, dy, dx)
+// ascending.
 __host__ __device__ constexpr int stencil_size(int dim, int m)
 {
     int idx = 0;
@@ -216,91 +101,13 @@ __host__ __device__ constexpr int stencil_size(int dim, int m)
     return idx;
 }
 
-// sqrt of a small non-negative integer, by Newton's method in double.
-__host__ __device__ constexpr double csqrt(double x)
-{
-    double r = x > 1.0 ? x : 1.0;
-    for (int i = 0; i < 64; ++i) r = 0.5 * (r + x / r);
-    return x == 0.0 ? 0.0 : r;
-}
-
 // Partial-volume factor in lattice units: (m + 1/2 - |d|) for |d| > m - 1/2.
 __host__ __device__ constexpr double vol_factor_lattice(int m, double r0)
 {
     return r0 > m - 0.5 ? (m + 0.5 - r0) : 1.0;
 }
 
-template <int DIM, int L>
-struct Brick {
-    static constexpr int bx = 1 << ((L + DIM - 1) / DIM);
-    static constexpr int by = 1 << ((L + DIM - 2) / DIM);
-    static constexpr int bz = DIM == 3 ? (1 << (L / 3)) : 1;
-    static constexpr int T = 1 << L;
-    static_assert(bx * by * bz == T, "brick");
-};
-
-// Compile-time halo-box geometry for horizon M.
-template <int DIM, int L, int M>
-struct Box {
-    using B = Brick<DIM, L>;
-    static constexpr int HX = B::bx + 2 * M;
-    static constexpr int HY = B::by + 2 * M;
-    static constexpr int HZ = DIM == 3 ? B::bz + 2 * M : 1;
-    static constexpr int N = HX * HY * HZ;
-};
-
-// Compile-time loop: f(std::integral_constant<int, K>) for K = 0..N-1.
-template <class F, int... Ks>
-__device__ __forceinline__ void static_for_impl(F &&f, std::integer_sequence<int, Ks...>)
-{
-    (f(std::integral_constant<int, Ks>{}), ...);
-}
-template <int N, class F>
-__device__ __forceinline__ void static_for(F &&f)
-{
-    static_for_impl(f, std::make_integer_sequence<int, N>{});
-}
-
 // --------------------------------------------------------------- staging
-
-// Local Morton code of brick-local coordinates (x, y, z) for a brick of 2^L codes.
-__device__ __forceinline__ int local_code(int dim, int x, int y, int z)
-{
-    return (int)morton_encode(dim, (uint32_t)x, (uint32_t)y, (uint32_t)z);
-}
-
-// Reference displacement of a tile as FP32 hi/lo (FP32C) or FP64.
-struct RefF { float3 hi, lo; };
-
-// The staging source of one step: 32 bytes per slot. FP32C: float4 hi, float4 lo;
-// FP64: double4_32a (x, y, z, 0).
-struct StageSrc {
-    const float4 *hl;      // FP32C
-    const double4_32a *d4;     // FP64
-};
-
-__device__ __forceinline__ float4 stage_fp32c(const float4 *hl, int slot, const RefF &ref, float inv_h)
-{
-    float4 hi = __ldg(&hl[2 * slot]);
-    float4 lo = __ldg(&hl[2 * slot + 1]);
-    float4 r;
-    r.x = ((hi.x - ref.hi.x) + (lo.x - ref.lo.x)) * inv_h;
-    r.y = ((hi.y - ref.hi.y) + (lo.y - ref.lo.y)) * inv_h;
-    r.z = ((hi.z - ref.hi.z) + (lo.z - ref.lo.z)) * inv_h;
-    r.w = 0.f;
-    return r;
-}
-
-__device__ __forceinline__ double4_32a stage_fp64(const double4_32a *d4, int slot, const double3 &ref, double inv_h)
-{
-    double4_32a a = d4[slot];
-    double4_32a r;
-    r.x = (a.x - ref.x) * inv_h;
-    r.y = (a.y - ref.y) * inv_h;
-    r.z = (a.z - ref.z) * inv_h;
-    r.w = 0.0;
-    return r;
-}
 
 // Global coordinates of box index b for a tile with origin org (runtime box dims).
 __device__ __forceinline__ void box_coord(int b, int HX, int HY, int m, int dim, const int4 &org,
