@@ -24,7 +24,8 @@
 // by dz = -3 alone, at dx = dy = 0, so it needs 8 rows of the 14 (m = 3: 1680 entries
 // of 1960, 67 instead of 78 KB for the LPS force pass, which lets three CTAs share an
 // SM instead of two), and of a column only the points within the horizon of the tile
-// are loaded (2104 instead of 2 x 1960 at m = 3).
+// are loaded (2104 instead of 2 x 1960 at m = 3). Where these passes run: rows_pmb,
+// rows_dil and rows_frc in pd_tile.cuh.
 #pragma once
 
 #include <string.h>

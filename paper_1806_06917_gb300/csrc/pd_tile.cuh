@@ -215,19 +215,21 @@ constexpr int SMS = 152;
 constexpr int PTAB_MIN_TILES = 2048;
 // Where the row-wise passes take over (us a step, word-wise and row-wise):
 // - PMB and the dilatation from two tiles per SM on (40^3 PMB, 125 tiles: 20.1 and 24.7; 64^3,
-//   512 tiles: 49.3 and 46.8). Below, the word-wise kernels have twice as many threads per
+//   512 tiles: 49.2 and 46.6). Below, the word-wise kernels have twice as many threads per
 //   tile.
-// - PMB at m = 3 (two ranges: 128^3 322 and 255). Shorter horizons leave segments of one and
-//   two bonds (m = 1: 128^3 96 and 110; m = 2: 80^3 32.3 and 33.9, 128^3 132 and 139), and at
-//   longer ones the word-wise kernel runs two threads a pair (m = 4: 64^3 88.7 and 99.6;
-//   m = 5: 169 and 176).
+// - PMB at m = 3 (128^3 277 and 247; summed in two ranges 329 and 261). Shorter horizons leave
+//   segments of one and two bonds (m = 1: 128^3 96.3 and 110; m = 2: 80 x 80 x 72 32.3 and 33.9,
+//   128^3 131 and 139), and at longer ones the word-wise kernel runs two threads a pair (m = 4:
+//   64^3 88.6 and 99.5; m = 5: 169 and 176).
 // - but not from 4.5 to 5 tiles per SM: the four CTAs of an SM end together here, so that the
-//   last tiles gather on a few SMs (693 tiles 60.4 and 60.0, 704 to 756 60.3 and 65.8, 768 69.6
-//   and 66.4).
-// - LPS from m = 2 on (m = 1: 56^3 0.94 of the speed, 128^3 0.98).
+//   last tiles gather on a few SMs (693 tiles 60.2 and 59.6, 704 to 756 60.2 and 65, 768 69.2
+//   and 66.1).
+// - the dilatation from m = 2 on (m = 1, LPS steps with the row-wise force: 56^3 25.2 and 26.9,
+//   128^3 185 and 196).
 // - the LPS force pass, at 128 registers and two CTAs per SM, from more than one tile per SM
 //   on (45 x 37 x 52, 210 tiles: 36.9 and 34.2; 33 x 45 x 27 with m = 4, 120 tiles: 38.9 and 42.7),
-//   where two CTAs' boxes fit in an SM (m = 5, one CTA: 48^3 210 and 227).
+//   where two CTAs' boxes fit in an SM (m = 5, one CTA: steps of 48^3 210 and 227, 56^3 292 and
+//   313).
 constexpr int ROWS_MIN_TILES = 2 * SMS, ROWS_MIN_TILES_FRC = SMS + 1;
 inline bool rows_pmb(const Geom &g)
 {
