@@ -17,12 +17,13 @@
 //   F  += w y                                                                 3 + 3
 // 28 in 3D and 23 in 2D (dilatation 23, LPS force 32, tangent product 45 and 36). The
 // quotient, the dilatation's root and 1 / sqrt(q) round once. 64^3 PMB step with breaking
-// 3.58 -> 1.67 ms (28 instructions a bond cost 1.45), 40^3 LPS step 1.70 -> 0.93 ms, 97^2
+// 3.58 -> 1.67 ms (28 instructions a bond cost 1.45), 40^3 LPS step 1.70 -> 0.88 ms, 97^2
 // NP step (m = 8; its exponential by a short series near 0) 2.06 -> 0.165 ms, tangent product
 // and force of the 200^2 plate through the torch bridge 0.556 -> 0.25 ms. The error against
 // extended precision is that of the templates, 1.3 to 5e-16 for m = 1 to 5 (relative L2), also
 // for compressed bonds (f64_len2).
 #include <algorithm>
+#include <type_traits>
 
 #include "pd_tile.cuh"
 
@@ -77,14 +78,27 @@ __device__ __forceinline__ double f64_exp_neg(double x)
 // |y|^2 of a bond with lattice vector d, |d|^2 = d2: num + d2, and y.y where a bond has
 // lost half of that and more. There the sum cancels (relative error 2^-53 d2 / |y|^2: 1e-12
 // at a hundredth of the length, and down to 0 or below for a collapsed bond); above, both
-// agree to the last bit or two. The high words are compared as integers and y.y stands out
-// of line, so that only the bonds concerned pay FP64 instructions (in line they were
-// predicated, and every bond paid: 64^3 PMB step 1.64 -> 1.81 ms).
+// agree to the last bit or two. High words are compared as integers, so that only the
+// bonds concerned pay FP64 instructions (y.y in line was predicated, and every bond paid:
+// 64^3 PMB step 1.64 -> 1.81 ms): in the PMB pass y.y stands out of line; the LPS passes and
+// the tangent product sum a mask word's bonds with num + d2, note whether one is so short,
+// and then sum the word once more with EXACT, which leaves the loop without a branch (40^3
+// LPS step 0.928 -> 0.880 ms against the call; PMB, whose breaking test is a call as it is, 64^3
+// with m = 4 3.48 -> 3.60).
+__device__ __forceinline__ bool f64_short(double q, double d2) { return __double2hiint(q) < __double2hiint(d2) - 0x100000; }
 __device__ __noinline__ double f64_dot(double x, double y, double z) { return fma(z, z, fma(y, y, x * x)); }
 __device__ __forceinline__ double f64_len2(double num, double d2, double yx, double yy, double yz)
 {
     const double q = num + d2;
-    return __double2hiint(q) < __double2hiint(d2) - 0x100000 ? f64_dot(yx, yy, yz) : q;
+    return f64_short(q, d2) ? f64_dot(yx, yy, yz) : q;
+}
+template <bool EXACT>
+__device__ __forceinline__ double f64_len2(double num, double d2, double yx, double yy, double yz, bool &low)
+{
+    double q = num + d2;
+    if (!EXACT) low = low || f64_short(q, d2);
+    else if (f64_short(q, d2)) q = fma(yz, yz, fma(yy, yy, yx * yx));
+    return q;
 }
 
 // ------------------------------------------------------------- bond-based
@@ -239,17 +253,29 @@ __global__ void __launch_bounds__(256) f64_lps_dil(const __grid_constant__ TileA
         for (int w = 0; w < g.W; ++w) {
             const uint32_t word = a.mask[(size_t)w * g.nslots + p.slot];
             const int nb = min(32, g.S - 32 * w);
-#pragma unroll 4
-            for (int b = 0; b < nb; ++b) {
-                if (!((word >> b) & 1u)) continue;
+            const double acc0 = acc;
+            bool low = false;
+            auto bond = [&](int b, auto exact) {
                 const F64Ent &e = tab[32 * w + b];
                 const double4_32a rj = box[p.bi + e.off];
                 const double ex = rj.x - ui.x, ey = rj.y - ui.y, ez = rj.z - ui.z;
                 const double num = f64_num3(e, ex, ey, ez);
-                const double q = f64_len2(num, e.d2, fma(0.5, e.dx, ex), fma(0.5, e.dy, ey), fma(0.5, e.dz, ez));
+                const double q = f64_len2<exact.value>(num, e.d2, fma(0.5, e.dx, ex), fma(0.5, e.dy, ey),
+                                                       fma(0.5, e.dz, ez), low);
                 double x = f64_div(num, f64_sqrt_rn(q) + e.R);
                 if (VOL) x *= e.C;
                 acc = fma(e.R, x, acc);
+            };
+#pragma unroll 4
+            for (int b = 0; b < nb; ++b) {
+                if (!((word >> b) & 1u)) continue;
+                bond(b, std::false_type());
+            }
+            if (low) {
+                acc = acc0;
+#pragma unroll 1
+                for (int b = 0; b < nb; ++b)
+                    if ((word >> b) & 1u) bond(b, std::true_type());
             }
         }
         a.theta64[p.slot] = 3.0 * acc / a.mtil[p.slot];
@@ -296,16 +322,16 @@ __global__ void __launch_bounds__(256) f64_lps_force(const __grid_constant__ Til
         for (int w = 0; w < g.W; ++w) {
             const uint32_t word = a.mask[(size_t)w * g.nslots + p.slot];
             const int nb = min(32, g.S - 32 * w);
-#pragma unroll 4
-            for (int b = 0; b < nb; ++b) {
-                if (!((word >> b) & 1u)) continue;
+            const double X0 = Fx, Y0 = Fy, Z0 = Fz;
+            bool low = false;
+            auto bond = [&](int b, auto exact) {
                 const F64Ent &e = tab[32 * w + b];
                 const int bj = p.bi + e.off;
                 const double4_32a rj = box[bj];
                 const double ex = rj.x - ui.x, ey = rj.y - ui.y, ez = rj.z - ui.z;
                 const double yx = fma(0.5, e.dx, ex), yy = fma(0.5, e.dy, ey), yz = fma(0.5, e.dz, ez);
                 const double num = f64_num3(e, ex, ey, ez);
-                const double q = f64_len2(num, e.d2, yx, yy, yz), rs = f64_rsqrt(q);
+                const double q = f64_len2<exact.value>(num, e.d2, yx, yy, yz, low), rs = f64_rsqrt(q);
                 const double x = f64_div(num, fma(q, rs, e.R));
                 double gg = e.R * (ui.w + rj.w);
                 gg = fma(x, bi + boxb[bj], gg);
@@ -314,6 +340,17 @@ __global__ void __launch_bounds__(256) f64_lps_force(const __grid_constant__ Til
                 Fx = fma(wgt, yx, Fx);
                 Fy = fma(wgt, yy, Fy);
                 Fz = fma(wgt, yz, Fz);
+            };
+#pragma unroll 4
+            for (int b = 0; b < nb; ++b) {
+                if (!((word >> b) & 1u)) continue;
+                bond(b, std::false_type());
+            }
+            if (low) {
+                Fx = X0, Fy = Y0, Fz = Z0;
+#pragma unroll 1
+                for (int b = 0; b < nb; ++b)
+                    if ((word >> b) & 1u) bond(b, std::true_type());
             }
         }
         const double f[3] = {a.inv_h * Fx, a.inv_h * Fy, a.inv_h * Fz};
@@ -363,9 +400,9 @@ __global__ void __launch_bounds__(256) f64_jvp(const __grid_constant__ TileArgs 
         for (int w = 0; w < g.W; ++w) {
             const uint32_t word = a.mask[(size_t)w * g.nslots + p.slot];
             const int nb = min(32, g.S - 32 * w);
-#pragma unroll 2
-            for (int b = 0; b < nb; ++b) {
-                if (!((word >> b) & 1u)) continue;
+            const double X0 = ox, Y0 = oy, Z0 = oz;
+            bool low = false;
+            auto bond = [&](int b, auto exact) {
                 const F64Ent &e = tab[32 * w + b];
                 const double4_32a uj = box[p.bi + e.off], wj = wbox[p.bi + e.off];
                 const double ex = uj.x - ui.x, ey = uj.y - ui.y;
@@ -383,7 +420,7 @@ __global__ void __launch_bounds__(256) f64_jvp(const __grid_constant__ TileArgs 
                 } else {
                     num = f64_num2(e, ex, ey);
                 }
-                const double q = f64_len2(num, e.d2, yx, yy, yz), rs = f64_rsqrt(q);
+                const double q = f64_len2<exact.value>(num, e.d2, yx, yy, yz, low), rs = f64_rsqrt(q);
                 const double cs = f64_div(num, fma(e.C, q * rs, e.R * q));         // V_ij s / r
                 const double cn = ndw * rs * (e.I - cs) * rs;                      // times y
                 // a bond's two terms first: added to the sum one by one they round it twice (an
@@ -391,6 +428,17 @@ __global__ void __launch_bounds__(256) f64_jvp(const __grid_constant__ TileArgs 
                 ox += fma(cn, yx, cs * dwx);
                 oy += fma(cn, yy, cs * dwy);
                 if (DIM == 3) oz += fma(cn, yz, cs * dwz);
+            };
+#pragma unroll 2
+            for (int b = 0; b < nb; ++b) {
+                if (!((word >> b) & 1u)) continue;
+                bond(b, std::false_type());
+            }
+            if (low) {
+                ox = X0, oy = Y0, oz = Z0;
+#pragma unroll 1
+                for (int b = 0; b < nb; ++b)
+                    if ((word >> b) & 1u) bond(b, std::true_type());
             }
         }
         a.jv[0][p.slot] = sc * ox;
